@@ -51,17 +51,15 @@ namespace {
 
 // Slabs per iteration of the middle range (plane_walk) and resident CTAs per
 // SM the register allocation targets, measured on GB300 (256^3 cube, 240
-// views of 512^2; 512^3 cube, 360 views of 1024^2): the static forward keeps
-// the loads of six slabs in flight (7.49 / 114.8 ms; four slabs 7.72 /
-// 129.9, seven 7.60 / 129.0, eight 7.53 / 124.1, twelve 7.44 / 122.7, all at
-// four CTAs; three slabs 7.78, five 8.09, two at five CTAs 10.5 on the 256^3
-// cube); the transpose, bound by the rate at which an SM sends reduction
+// views of 512^2): the static forward keeps the loads of five slabs in
+// flight (6.92 ms; four slabs 7.21, six 7.00, eight 7.26, four at five CTAs
+// 7.14); the transpose, bound by the rate at which an SM sends reduction
 // sectors to L2, walks one slab per iteration at six CTAs (9.19 ms; five
 // CTAs 9.31, two slabs per iteration 9.52).
-constexpr int kFwdUnroll = 6;
-// bf16 cubes: eight slabs (7.97 / 109.4 ms against 8.11 / 112.0 at six; the
-// predicated slot bodies 9.01 / 125.0)
-constexpr int kFwdBf16Unroll = 8;
+constexpr int kFwdUnroll = 5;
+// bf16 cubes: six slabs (512^3 cube, 48 views of 1024^2: 14.24 ms; eight
+// slabs 14.47, four at five CTAs 14.53)
+constexpr int kFwdBf16Unroll = 6;
 constexpr int kFwdTimeUnroll = 1;
 constexpr int kFwdMinBlocks = 4;
 constexpr int kAdjUnroll = 1;
