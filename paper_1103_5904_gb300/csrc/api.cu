@@ -52,6 +52,28 @@ tomo_status ensure(tomo_ctx *ctx, DevBuf &b, size_t bytes)
     return TOMO_OK;
 }
 
+// ensure() for a buffer that the gathering walks address by units of `unit`
+// bytes: a new allocation with a unit across a multiple of 2^32 (near_buffers)
+// is tried once more elsewhere.  Only speed depends on the outcome.
+static tomo_status ensure_near(tomo_ctx *ctx, DevBuf &b, size_t bytes, size_t unit)
+{
+    if (b.bytes >= bytes && b.p) return TOMO_OK;
+    tomo_status st = ensure(ctx, b, bytes);
+    if (st || unit == 0 || near_buffers(b.p, unit, (int)(bytes / unit))) return st;
+    void *p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return TOMO_OK;
+    }
+    void *drop = p;
+    if (near_buffers(p, unit, (int)(bytes / unit))) {
+        drop = b.p;
+        b.p = p;
+    }
+    CUDA_TRY(ctx, cudaFree(drop));
+    return TOMO_OK;
+}
+
 bool finite_all(const double *v, int n)
 {
     for (int i = 0; i < n; ++i)
@@ -358,7 +380,9 @@ tomo_status ensure_plane(tomo_ctx *ctx, const tomo_cube_geom *c,
     const size_t bytes =
         sizeof(float) * (size_t)c->nx * c->ny * c->nz * (size_t)n_frames;
     tomo_status st;
-    if ((st = ensure(ctx, ctx->lay1, bytes)) || (st = ensure(ctx, ctx->lay2, bytes)))
+    const size_t unit = bytes / (size_t)n_frames;
+    if ((st = ensure_near(ctx, ctx->lay1, bytes, unit)) ||
+        (st = ensure_near(ctx, ctx->lay2, bytes, unit)))
         return st;
     return TOMO_OK;
 }
@@ -372,7 +396,7 @@ tomo_status ensure_pairs(tomo_ctx *ctx, const tomo_cube_geom *c,
     const size_t bytes = 8 * (size_t)c->nx * c->ny * c->nz * npairs;
     tomo_status st;
     for (int L = 0; L < 3; ++L)
-        if ((st = ensure(ctx, ctx->pr[L], bytes))) return st;
+        if ((st = ensure_near(ctx, ctx->pr[L], bytes, bytes / npairs))) return st;
     return TOMO_OK;
 }
 
@@ -452,7 +476,7 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
                                   per_ray_list(ctx), ctx->num_sms));
         LAUNCH(ctx, TOMO_K_FORWARD, s,
                launch_forward_plane_pair(
-                   rays, prm, pc, cube_dev, dtype, fstride, mask, out,
+                   rays, prm, pc, n_frames - 1, cube_dev, dtype, fstride, mask, out,
                    g->n_img, g->nu, g->nv, c, done, s, !all,
                    plane_group(ctx, c, g, false, 8 * fstride * (n_frames - 1),
                                n_frames - 1)));

@@ -50,24 +50,36 @@ namespace tomo {
 namespace {
 
 // Slabs per iteration of the middle range (plane_walk) and resident CTAs per
-// SM the register allocation targets, measured on GB300 (256^3 cube, 240
-// views of 512^2): the static forward keeps the loads of five slabs in
-// flight (6.92 ms; four slabs 7.21, six 7.00, eight 7.26, four at five CTAs
-// 7.14); the transpose, bound by the rate at which an SM sends reduction
-// sectors to L2, walks one slab per iteration at six CTAs (9.19 ms; five
-// CTAs 9.31, two slabs per iteration 9.52).
-constexpr int kFwdUnroll = 5;
-// bf16 cubes: six slabs (512^3 cube, 48 views of 1024^2: 14.24 ms; eight
-// slabs 14.47, four at five CTAs 14.53)
-constexpr int kFwdBf16Unroll = 6;
+// SM the register allocation targets, measured on GB300.  The static forward
+// by address of a float cube (256^3, 240 views of 512^2) keeps the loads of
+// five slabs in flight at five CTAs: 6.30 ms (six slabs 6.44, eight 6.39,
+// four 6.40, three 6.80; six CTAs with four slabs 6.38, with three 7.24; four
+// CTAs with six slabs 6.45); of a bf16 cube (512^3, 48 views of 1024^2) four
+// slabs at six CTAs: 12.53 ms (five CTAs with four to eight slabs
+// 12.94-13.14).  By offset, for a buffer across a multiple of 2^32: 6.92 and
+// 14.2 ms at four CTAs with five and six slabs.  The transpose, bound by the
+// rate at which an SM sends reduction sectors to L2, walks one slab per
+// iteration at six CTAs (9.19 ms; five CTAs 9.31, two slabs per iteration
+// 9.52).
+template <typename CubeT, bool kNear>
+struct FwdShape {
+    static constexpr int kUnroll = sizeof(CubeT) == 2 ? 6 : 5, kMinBlocks = 4;
+};
+template <>
+struct FwdShape<float, true> {
+    static constexpr int kUnroll = 5, kMinBlocks = 5;
+};
+template <>
+struct FwdShape<uint16_t, true> {
+    static constexpr int kUnroll = 4, kMinBlocks = 6;
+};
 constexpr int kFwdTimeUnroll = 1;
-constexpr int kFwdMinBlocks = 4;
 constexpr int kAdjUnroll = 1;
 constexpr int kAdjMinBlocks = 6;
 constexpr int kAdjTimeMinBlocks = 5;
 
-template <typename CubeT, bool kTime>
-__global__ void __launch_bounds__(256, kFwdMinBlocks)
+template <typename CubeT, bool kTime, bool kNear>
+__global__ void __launch_bounds__(256, FwdShape<CubeT, kNear>::kMinBlocks)
 k_forward_plane(const RayRec *__restrict__ rays,
                 const ImgParam *__restrict__ prm, PlaneCubes cubes,
                 int64_t frame_stride, const uint8_t *__restrict__ mask,
@@ -116,11 +128,10 @@ k_forward_plane(const RayRec *__restrict__ rays,
             acc = op2.acc;
         }
     } else {
-        PlaneGatherOp<CubeT> op;
+        PlaneGatherOp<CubeT, kNear> op;
         op.c = lay;
         op.acc = 0.0f;
-        constexpr int kU = sizeof(CubeT) == 2 ? kFwdBf16Unroll : kFwdUnroll;
-        plane_walk_for<kU>(q.pad, p, regular, op);
+        plane_walk_for<FwdShape<CubeT, kNear>::kUnroll>(q.pad, p, regular, op);
         acc = op.acc;
         if (live && !regular) {
             GatherOp<CubeT> op2;
@@ -383,24 +394,31 @@ cudaError_t launch_forward_plane(const RayRec *rays, const ImgParam *prm,
     const dim3 grid = plane_grid(nu, nv, n_img, group);
     const int block = t.tile_u * t.tile_v;
     const bool om = only_marked;
+    const uint64_t c_bytes =
+        (uint64_t)c->nx * c->ny * c->nz * (dtype == TOMO_BF16 ? 2 : 4);
+    const bool near = !time_interp &&
+                      near_buffers(cubes.c[0], c_bytes) &&
+                      near_buffers(cubes.c[1], c_bytes) &&
+                      near_buffers(cubes.c[2], c_bytes);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, block, 0, s>>>(rays, prm, cubes, frame_stride, mask, out,
+                                      nu, nv, c->nx, c->ny, c->nz, t, done, om,
+                                      n_img, group);
+    };
     if (dtype == TOMO_BF16) {
         if (time_interp)
-            k_forward_plane<uint16_t, true><<<grid, block, 0, s>>>(
-                rays, prm, cubes, frame_stride, mask, out, nu, nv, c->nx,
-                c->ny, c->nz, t, done, om, n_img, group);
+            launch(k_forward_plane<uint16_t, true, false>);
+        else if (near)
+            launch(k_forward_plane<uint16_t, false, true>);
         else
-            k_forward_plane<uint16_t, false><<<grid, block, 0, s>>>(
-                rays, prm, cubes, frame_stride, mask, out, nu, nv, c->nx,
-                c->ny, c->nz, t, done, om, n_img, group);
+            launch(k_forward_plane<uint16_t, false, false>);
     } else {
         if (time_interp)
-            k_forward_plane<float, true><<<grid, block, 0, s>>>(
-                rays, prm, cubes, frame_stride, mask, out, nu, nv, c->nx,
-                c->ny, c->nz, t, done, om, n_img, group);
+            launch(k_forward_plane<float, true, false>);
+        else if (near)
+            launch(k_forward_plane<float, false, true>);
         else
-            k_forward_plane<float, false><<<grid, block, 0, s>>>(
-                rays, prm, cubes, frame_stride, mask, out, nu, nv, c->nx,
-                c->ny, c->nz, t, done, om, n_img, group);
+            launch(k_forward_plane<float, false, false>);
     }
     return cudaGetLastError();
 }

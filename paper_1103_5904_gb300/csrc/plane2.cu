@@ -30,14 +30,16 @@ namespace tomo {
 
 namespace {
 
-// Slabs per iteration of the forward's middle range (loads in flight), as
-// measured on GB300: 8-frame 256^3 temporal P 22.7 ms at 2 slabs, 16.6 ms
-// at 4, 18.6 ms at 6, 20.7 ms at 8 (3 CTAs per SM); Thomson B forward on
-// the 256^3 cube 14.8, 11.6, 12.5, 13.2 ms.  At 4 CTAs per SM with byte
-// offsets: temporal 15.9 ms at 4 slabs, 17.1 at 6, 15.7 at 8; B 10.9, 12.1,
-// 11.3 ms.
+// Slabs per iteration of the forward's middle range (loads in flight) and
+// CTAs per SM, measured on GB300.  By address (near_buffers): P and P^T of 8
+// frames (256^3, 120 views of 512^2) with 4 / 5 / 6 / 7 / 8 slabs of P 20.9
+// (five CTAs) / 20.27 / 20.15 / 20.13 / 20.03 ms, by offset with four slabs
+// 20.63; Thomson B (256^3, 90 views) 9.67 / 8.91 / 9.00 / 8.93 / 8.83 ms, by
+// offset 9.57.
 constexpr int kPairFwdUnroll = 4;
 constexpr int kPairFwdMinBlocks = 4;
+constexpr int kPairNearUnroll = 8;
+constexpr int kBNearUnroll = 8;
 constexpr int kPairAdjMinBlocks = 5;
 
 __device__ __forceinline__ float2 load_pair(const float2 *c, int idx)
@@ -78,13 +80,26 @@ __device__ __forceinline__ float *pick(const PlaneAcc &c, int L)
     return L == 1 ? c.c[1] : (L == 2 ? c.c[2] : c.c[0]);
 }
 
-// Plane ops (byte offsets, see plane.cuh)
-template <typename PairT>
+// Plane ops (see plane.cuh; kNear: gathers by address)
+template <typename PairT, bool kNearBuf = false>
 struct PlaneGatherPairOp {
     const PairT *c;
     float w0, w1, acc;
     using Val = float2;
     static constexpr bool kAllSlots = true;
+    static constexpr bool kNear = kNearBuf;
+    __device__ __forceinline__ const char *at(uint32_t off) const
+    {
+        return reinterpret_cast<const char *>(c) + off;
+    }
+    __device__ __forceinline__ uint32_t off(const char *p) const
+    {
+        return (uint32_t)(p - reinterpret_cast<const char *>(c));
+    }
+    __device__ __forceinline__ float2 load(const char *p) const
+    {
+        return load_pair(reinterpret_cast<const PairT *>(p), 0);
+    }
     __device__ __forceinline__ void clear() { acc = 0.0f; }
     __device__ __forceinline__ float2 fetch(bool on, uint32_t off) const
     {
@@ -100,13 +115,27 @@ struct PlaneGatherPairOp {
     }
 };
 
+template <bool kNearBuf = false>
 struct PlaneGatherBOp {
     const float2 *c;
     float s1, s2;
     using Val = float2;
-    // two sums per slot: the predicated bodies measured faster (11.0
-    // against 12.9 ms on the 256^3 cube)
-    static constexpr bool kAllSlots = false;
+    // by offset, the predicated bodies measured faster (two sums per slot:
+    // 11.0 against 12.9 ms on the 256^3 cube)
+    static constexpr bool kAllSlots = kNearBuf;
+    static constexpr bool kNear = kNearBuf;
+    __device__ __forceinline__ const char *at(uint32_t off) const
+    {
+        return reinterpret_cast<const char *>(c) + off;
+    }
+    __device__ __forceinline__ uint32_t off(const char *p) const
+    {
+        return (uint32_t)(p - reinterpret_cast<const char *>(c));
+    }
+    __device__ __forceinline__ float2 load(const char *p) const
+    {
+        return load_pair(reinterpret_cast<const float2 *>(p), 0);
+    }
     __device__ __forceinline__ void clear()
     {
         s1 = 0.0f;
@@ -156,6 +185,7 @@ struct PlaneScatterPairOp {
     float y0, y1;
     using Val = NoVal;
     static constexpr bool kAllSlots = false;
+    static constexpr bool kNear = false;
     __device__ __forceinline__ NoVal fetch(bool, uint32_t) const { return NoVal(); }
     __device__ __forceinline__ void apply(bool on, uint32_t off, float len, NoVal)
     {
@@ -181,7 +211,7 @@ struct ScatterPairOp {
 // Time-interpolated forward on frame pairs.  pairs.c[L]: pair buffer of
 // layout L, T - 1 pairs of n voxels; native: the caller's frames (for rays
 // outside the plane walk).
-template <typename CubeT, typename PairT>
+template <typename CubeT, typename PairT, bool kNear>
 __global__ void __launch_bounds__(256, kPairFwdMinBlocks)
 k_forward_plane_pair(const RayRec *__restrict__ rays,
                      const ImgParam *__restrict__ prm, PlaneCubes pairs,
@@ -207,12 +237,12 @@ k_forward_plane_pair(const RayRec *__restrict__ rays,
     const bool regular = live && plane_ray(r, q.pad, nx, ny, nz, p, sizeof(PairT));
     const int L = (q.pad >> 2) & 3;
     const int64_t f0 = (int64_t)img_frame(q) * fstride;
-    PlaneGatherPairOp<PairT> op;
+    PlaneGatherPairOp<PairT, kNear> op;
     op.c = static_cast<const PairT *>(pick(pairs, L)) + f0;
     op.w0 = q.w0;
     op.w1 = q.w;
     op.acc = 0.0f;
-    plane_walk_for<kPairFwdUnroll>(q.pad, p, regular, op);
+    plane_walk_for<kNear ? kPairNearUnroll : kPairFwdUnroll>(q.pad, p, regular, op);
     float acc = op.acc;
     if (live && !regular) {
         GatherTimeOp<CubeT> op2;
@@ -232,6 +262,7 @@ k_forward_plane_pair(const RayRec *__restrict__ rays,
 // walks every image plane by plane, 1 the images whose hint has the
 // plane-forward bit, 0 none; the other images (and the rays that do not fit
 // the plane walk) walk per ray on the native pairs.
+template <bool kNear>
 __global__ void __launch_bounds__(256, kPairFwdMinBlocks)
 k_forward_b(const RayRec *__restrict__ rays, const ImgParam *__restrict__ prm,
             PlaneCubes pairs, const float *__restrict__ rho2,
@@ -259,11 +290,11 @@ k_forward_b(const RayRec *__restrict__ rays, const ImgParam *__restrict__ prm,
     const int L = (q.pad >> 2) & 3;
     float s1 = 0.0f, s2 = 0.0f;
     if (plane) {
-        PlaneGatherBOp op;
+        PlaneGatherBOp<kNear> op;
         op.c = static_cast<const float2 *>(pick(pairs, L));
         op.s1 = 0.0f;
         op.s2 = 0.0f;
-        plane_walk_for<kPairFwdUnroll>(q.pad, p, regular, op);
+        plane_walk_for<kNear ? kBNearUnroll : kPairFwdUnroll>(q.pad, p, regular, op);
         s1 = op.s1;
         s2 = op.s2;
     }
@@ -668,7 +699,8 @@ cudaError_t launch_add_b_layout(const void *acc, void *out, int L,
 }
 
 cudaError_t launch_forward_plane_pair(const RayRec *rays, const ImgParam *prm,
-                                      PlaneCubes pairs, const void *native,
+                                      PlaneCubes pairs, int n_pairs,
+                                      const void *native,
                                       tomo_dtype dtype, int64_t fstride,
                                       const uint8_t *mask, float *out,
                                       int32_t n_img, int32_t nu, int32_t nv,
@@ -678,16 +710,24 @@ cudaError_t launch_forward_plane_pair(const RayRec *rays, const ImgParam *prm,
 {
     if (n_img <= 0) return cudaSuccess;
     const dim3 grid = plane_grid2(nu, nv, n_img, group);
-    if (dtype == TOMO_BF16)
-        k_forward_plane_pair<uint16_t, uint32_t><<<grid, 256, 0, s>>>(
-            rays, prm, pairs, static_cast<const uint16_t *>(native), fstride,
-            mask, out, nu, nv, c->nx, c->ny, c->nz, kPlaneTiling2, done,
-            only_marked, n_img, group);
-    else
-        k_forward_plane_pair<float, float2><<<grid, 256, 0, s>>>(
-            rays, prm, pairs, static_cast<const float *>(native), fstride,
-            mask, out, nu, nv, c->nx, c->ny, c->nz, kPlaneTiling2, done,
-            only_marked, n_img, group);
+    const uint64_t bytes = (uint64_t)fstride * (dtype == TOMO_BF16 ? 4 : 8);
+    const bool near = near_buffers(pairs.c[0], bytes, n_pairs) &&
+                      near_buffers(pairs.c[1], bytes, n_pairs) &&
+                      near_buffers(pairs.c[2], bytes, n_pairs);
+    auto launch = [&](auto kernel, auto cube) {
+        kernel<<<grid, 256, 0, s>>>(rays, prm, pairs, cube, fstride, mask, out,
+                                    nu, nv, c->nx, c->ny, c->nz, kPlaneTiling2,
+                                    done, only_marked, n_img, group);
+    };
+    if (dtype == TOMO_BF16) {
+        const uint16_t *x = static_cast<const uint16_t *>(native);
+        if (near) launch(k_forward_plane_pair<uint16_t, uint32_t, true>, x);
+        else launch(k_forward_plane_pair<uint16_t, uint32_t, false>, x);
+    } else {
+        const float *x = static_cast<const float *>(native);
+        if (near) launch(k_forward_plane_pair<float, float2, true>, x);
+        else launch(k_forward_plane_pair<float, float2, false>, x);
+    }
     return cudaGetLastError();
 }
 
@@ -717,9 +757,17 @@ cudaError_t launch_forward_b(const RayRec *rays, const ImgParam *prm,
 {
     if (n_img <= 0) return cudaSuccess;
     const dim3 grid = plane_grid2(nu, nv, n_img, group);
-    k_forward_b<<<grid, 256, 0, s>>>(
-        rays, prm, pairs, rho2, mask, out, nu, nv, c->nx, c->ny, c->nz,
-        kPlaneTiling2, done, plane_mode, n_img, group);
+    const uint64_t bytes = 8 * (uint64_t)c->nx * c->ny * c->nz;
+    const bool near = near_buffers(pairs.c[0], bytes) &&
+                      near_buffers(pairs.c[1], bytes) &&
+                      near_buffers(pairs.c[2], bytes);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, 256, 0, s>>>(rays, prm, pairs, rho2, mask, out, nu, nv,
+                                    c->nx, c->ny, c->nz, kPlaneTiling2, done,
+                                    plane_mode, n_img, group);
+    };
+    if (near) launch(k_forward_b<true>);
+    else launch(k_forward_b<false>);
     return cudaGetLastError();
 }
 

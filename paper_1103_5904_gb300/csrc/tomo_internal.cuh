@@ -182,6 +182,16 @@ bool plane_supported(const tomo_cube_geom *c, int esize);
 // Images per group of the plane walks' CTA order (plane_cta in plane.cuh),
 // clamped to [1, n_img] and to the grid's y extent (tiles_v tile rows).
 int plane_group_clamp(int group, int n_img, int tiles_v);
+// Whether each of n consecutive buffers of `bytes` bytes at p lies between two
+// multiples of 2^32 (true for p NULL): the gathering plane walks then keep a
+// voxel's address in a register pair of which only the low half changes.
+inline bool near_buffers(const void *p, uint64_t bytes, int n = 1)
+{
+    const uint64_t a = (uint64_t)(uintptr_t)p;
+    for (int k = 0; p != nullptr && k < n; ++k)
+        if (((a + k * bytes) >> 32) != ((a + (k + 1) * bytes - 1) >> 32)) return false;
+    return true;
+}
 // (copies for the forward: runs when bit `bit` of *used is set)
 cudaError_t launch_to_layout(const void *cube, tomo_dtype dtype, void *out,
                              int L, const tomo_cube_geom *c, int32_t n_frames,
@@ -310,7 +320,8 @@ cudaError_t launch_add_b_layout(const void *acc, void *out, int L,
                                 const tomo_cube_geom *c, const unsigned *used,
                                 const double *done, cudaStream_t s);
 cudaError_t launch_forward_plane_pair(const RayRec *rays, const ImgParam *prm,
-                                      PlaneCubes pairs, const void *native,
+                                      PlaneCubes pairs, int n_pairs,
+                                      const void *native,
                                       tomo_dtype dtype, int64_t fstride,
                                       const uint8_t *mask, float *out,
                                       int32_t n_img, int32_t nu, int32_t nv,
