@@ -908,7 +908,7 @@ tomo_status tomo_solve_batched(tomo_ctx *ctx, int32_t n,
             (st = ensure(ctx, P->timg, sizeof(float) * (poff[n] > 0 ? poff[n] : 1))) ||
             (st = ensure(ctx, P->S, sizeof(double) * n * (S_NSLOTS + stride))) ||
             (st = ensure(ctx, P->partials, sizeof(double) * 2 * max_items)) ||
-            (st = ensure(ctx, P->counters, sizeof(unsigned long long) * n_walks)))
+            (st = ensure(ctx, P->counters, sizeof(unsigned long long) * (n_walks + n))))
             return st;
         float *vb = (float *)P->vec.p, *vr = vb + NV, *vp = vr + NV, *vq = vp + NV;
         float *tim = (float *)P->timg.p;
@@ -1071,42 +1071,36 @@ tomo_status tomo_solve_batched(tomo_ctx *ctx, int32_t n,
                                     ctr + next_ctr++, wgrid, c));            \
         }                                                                    \
     } while (0)
-        e = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * n_walks, c);
+        // the queue counters and, behind them, one item counter per problem
+        unsigned *pc = (unsigned *)(ctr + n_walks);
+        e = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * (n_walks + n), c);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(S, 0, sizeof(double) * n * S_NSLOTS, c);
         CAP(TOMO_K_VECTOR, launch_fill_f64(rep, NAN, (int64_t)(n * stride), c));
-        CAP(TOMO_K_VECTOR, launch_vec_batched(BV_SUMSQ, V, pix_pre, n, warm, part,
-                                              vgrid, c));
-        CAP(TOMO_K_VECTOR, launch_finalize_batched(BV_SUMSQ, V, pix_pre, n, 0.0,
-                                                   part, c));
-        CAP(TOMO_K_VECTOR, launch_vec_batched(BV_ZERO, V, vox_pre, n, warm, part,
-                                              vgrid, c));
+        CAP(TOMO_K_VECTOR, launch_vec_batched(BV_SUMSQ, V, pix_pre, n, warm, 0.0,
+                                              part, pc, vgrid, c));
+        CAP(TOMO_K_VECTOR, launch_vec_batched(BV_ZERO, V, vox_pre, n, warm, 0.0,
+                                              part, pc, vgrid, c));
         CAP_ADJ(0, 0);
         if (warm) {
             CAP(TOMO_K_PRIOR, launch_vec_batched(BV_PRIOR_X, V, vox_pre, n, warm,
-                                                 part, vgrid, c));
+                                                 0.0, part, pc, vgrid, c));
             CAP_FWD(1, 0);
             CAP_ADJ(2, 1);
         }
-        CAP(TOMO_K_VECTOR, launch_vec_batched(BV_INIT, V, vox_pre, n, warm, part,
-                                              vgrid, c));
-        CAP(TOMO_K_VECTOR, launch_finalize_batched(BV_INIT, V, vox_pre, n, 0.0,
-                                                   part, c));
+        CAP(TOMO_K_VECTOR, launch_vec_batched(BV_INIT, V, vox_pre, n, warm, 0.0,
+                                              part, pc, vgrid, c));
         for (int32_t k = 0; k < n_iter; ++k) {
             CAP_FWD(3, 1);
             CAP(TOMO_K_PRIOR, launch_vec_batched(BV_PRIOR, V, vox_pre, n, warm,
-                                                 part, vgrid, c));
+                                                 0.0, part, pc, vgrid, c));
             CAP_ADJ(4, 2);
             CAP(TOMO_K_VECTOR, launch_vec_batched(BV_PQ, V, vox_pre, n, warm,
-                                                  part, vgrid, c));
-            CAP(TOMO_K_VECTOR, launch_finalize_batched(BV_PQ, V, vox_pre, n, 0.0,
-                                                       part, c));
+                                                  0.0, part, pc, vgrid, c));
             CAP(TOMO_K_VECTOR, launch_vec_batched(BV_UPDATE, V, vox_pre, n, warm,
-                                                  part, vgrid, c));
-            CAP(TOMO_K_VECTOR, launch_finalize_batched(BV_UPDATE, V, vox_pre, n,
-                                                       0.0, part, c));
+                                                  0.0, part, pc, vgrid, c));
             CAP(TOMO_K_VECTOR, launch_vec_batched(BV_DIR, V, vox_pre, n, warm,
-                                                  part, vgrid, c));
+                                                  0.0, part, pc, vgrid, c));
         }
 #undef CAP_ADJ
 #undef CAP_FWD

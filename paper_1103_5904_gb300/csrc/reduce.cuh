@@ -65,19 +65,34 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Sum over the CTA; valid in thread 0.  Ends with a barrier so `sm` (32
-// doubles of shared memory) can be reused by the next call.
-__device__ __forceinline__ double block_sum(double v, double *sm)
+// Sums of K values per thread over the CTA of 256 threads; total[] is valid in
+// thread 0.  GB300 completes about two FP64 operations per clock per SM, so a
+// warp-wide addition holds that pipe for 16 clocks: the CTA's values go
+// through shared memory and warp k adds up value k of all threads (7 + 5
+// warp-wide additions instead of 5 in each of 8 warps and 5 more).  Ends with
+// a barrier so `sm` can be reused by the next call.
+constexpr int kSumThreads = 256;
+
+template <int K>
+__device__ __forceinline__ void block_sums(const double (&v)[K], double (&total)[K],
+                                           double (*sm)[kSumThreads])
 {
-    v = warp_sum(v);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sm[w] = v;
+#pragma unroll
+    for (int k = 0; k < K; ++k) sm[k][threadIdx.x] = v[k];
     __syncthreads();
-    const int nw = blockDim.x >> 5;
-    v = (threadIdx.x < nw) ? sm[threadIdx.x] : 0.0;
-    if (w == 0) v = warp_sum(v);
+    if (w < K) {
+        double s = sm[w][lane];
+#pragma unroll
+        for (int i = 1; i < kSumThreads / 32; ++i) s += sm[w][lane + 32 * i];
+        s = warp_sum(s);
+        __syncwarp();
+        if (lane == 0) sm[w][0] = s;
+    }
     __syncthreads();
-    return v;
+#pragma unroll
+    for (int k = 0; k < K; ++k) total[k] = sm[k][0];
+    __syncthreads();
 }
 
 // Scalar steps; called by one thread with the grid-wide sums.

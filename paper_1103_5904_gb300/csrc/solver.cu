@@ -35,11 +35,12 @@ template <int K>
 __device__ bool grid_sum(double (&v)[K], double *partials,
                          unsigned int *counter, double (&total)[K])
 {
-    __shared__ double sm[32];
+    static_assert(kThreads == kSumThreads, "one value per thread");
+    __shared__ double sm[K][kSumThreads];
     __shared__ bool last;
-    for (int k = 0; k < K; ++k) v[k] = block_sum(v[k], sm);
+    block_sums<K>(v, total, sm);
     if (threadIdx.x == 0) {
-        for (int k = 0; k < K; ++k) partials[blockIdx.x * K + k] = v[k];
+        for (int k = 0; k < K; ++k) partials[blockIdx.x * K + k] = total[k];
         __threadfence();
         const unsigned int prev = atomicAdd(counter, 1u);
         last = (prev == gridDim.x - 1);
@@ -47,12 +48,11 @@ __device__ bool grid_sum(double (&v)[K], double *partials,
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    for (int k = 0; k < K; ++k) {
-        double s = 0.0;
-        for (unsigned int i = threadIdx.x; i < gridDim.x; i += blockDim.x)
-            s += __ldcg(partials + i * K + k);
-        total[k] = block_sum(s, sm);
-    }
+    double s[K];
+    for (int k = 0; k < K; ++k) s[k] = 0.0;
+    for (unsigned int i = threadIdx.x; i < gridDim.x; i += blockDim.x)
+        for (int k = 0; k < K; ++k) s[k] += __ldcg(partials + i * K + k);
+    block_sums<K>(s, total, sm);
     if (threadIdx.x == 0) *counter = 0u;
     return true;
 }
