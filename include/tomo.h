@@ -141,7 +141,8 @@ typedef struct tomo_ctx tomo_ctx;
                                   on every image; bit 2 for P on the images
                                   where it measured faster: views within
                                   ~1 degree of a cube-axis plane, or pixels
-                                  at least 0.75 voxel apart (per ray on the
+                                  at least 0.75 voxel apart (0.5 on cubes of
+                                  at least 2^20 voxels; per ray on the
                                   others).  A set bit
                                   makes the rays of a warp walk the cube one
                                   plane of the image's major axis at a time,
@@ -392,8 +393,9 @@ typedef struct {
     double min_pitch;      /* plane-synchronous walks when pitch >= this,
                               per-ray walks below (default 0.16) */
     double fwd_min_pitch;  /* P plane-synchronous when pitch >= this ... */
-    double fwd_max_ratio;  /* ... or ratio < this (defaults 0.75, 0.02; P
-                              per ray otherwise) */
+    double fwd_max_ratio;  /* ... or ratio < this (defaults 0.75, or 0.5
+                              for cubes of at least 2^20 voxels, and 0.02;
+                              P per ray otherwise) */
     double general_ratio;  /* plane walks cross every slab with the general
                               three-segment body when ratio >= this, else
                               they count the slabs to the next crossing of

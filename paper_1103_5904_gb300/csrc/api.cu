@@ -338,7 +338,7 @@ tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
         if (t.nx == c->nx && t.ny == c->ny && t.nz == c->nz && t.nu == g->nu &&
             t.nv == g->nv)
             return t.rules;
-    return ctx->rules;
+    return ctx->rules_set ? ctx->rules : default_plane_rules(*c);
 }
 
 // The device's rules (setup.cu) evaluated from the boresight, with margins

@@ -774,7 +774,14 @@ tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
     if ((cube == nullptr) != (img == nullptr))
         return fail(ctx, TOMO_ERR_ARG, "cube and img must both be given or "
                                        "both be NULL");
-    const tomo_plane_rules r = rules ? *rules : default_plane_rules();
+    if (!cube && !rules) {
+        ctx->rules_set = false;
+        return TOMO_OK;
+    }
+    tomo_status st;
+    if (cube && ((st = check_cube(ctx, cube, 1)) || (st = check_img(ctx, img))))
+        return st;
+    const tomo_plane_rules r = rules ? *rules : default_plane_rules(*cube);
     const double v[6] = { r.min_pitch, r.fwd_min_pitch, r.fwd_max_ratio,
                           r.general_ratio, r.fwd_group, r.adj_group };
     for (double x : v)
@@ -782,11 +789,9 @@ tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
             return fail(ctx, TOMO_ERR_ARG, "plane rules must be >= 0");
     if (!cube) {
         ctx->rules = r;
+        ctx->rules_set = true;
         return TOMO_OK;
     }
-    tomo_status st;
-    if ((st = check_cube(ctx, cube, 1)) || (st = check_img(ctx, img)))
-        return st;
     Tuned *e = bucket_of(ctx, cube, img);
     if (!e) {
         Tuned t;

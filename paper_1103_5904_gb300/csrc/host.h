@@ -51,8 +51,10 @@ struct tomo_ctx {
     // side; bit 1: Thomson B in one walk on (m' x, m x) pairs
     int channels = 3;
     tomo::Tiling tiling = { 32, 8, 8 };
-    // walk rules of size buckets without their own
-    tomo_plane_rules rules = tomo::default_plane_rules();
+    // walk rules of size buckets without their own, once set by the caller
+    // (else the built-in defaults of the bucket's cube)
+    tomo_plane_rules rules = {};
+    bool rules_set = false;
     // geometry cache
     bool key_valid = false;
     uint64_t key = 0;       // geometry of the cached ray records

@@ -69,19 +69,29 @@ constexpr double kPlaneMinPitch = 0.16;
 //    loop when lo < kPlaneFwdMaxRatio (0.81x the per-ray forward at lo = 0,
 //    0.94x at 0.017, 1.04x at 0.026), and whenever the pixels are at least
 //    kPlaneFwdMinPitch voxels apart, where the per-ray warps share few L1
-//    lines (1.22 against 2.14 ms at 1.07 voxel).
+//    lines (1.22 against 2.14 ms at 1.07 voxel); from kPlaneLargeCube voxels
+//    on kPlaneFwdMinPitchLarge.  Per-ray over plane time of the every-slab
+//    body at 2 / 7 / 30 degrees of latitude: pixels 0.53 voxel apart, 64^3
+//    cube 0.91 / 0.92 / 1.21 (bf16 0.87 / 0.91 / 1.13), 128^3 1.08 / 1.18 /
+//    1.49 (0.99 / 1.09 / 1.38), 256^3 1.35 / 1.42 / 1.79 (1.21 / 1.28 / 1.60);
+//    0.35 apart, 128^3 0.96 / 1.05 / 1.34 (0.86 / 0.94 / 1.21); 0.8 apart,
+//    64^3 1.15 / 1.16 / 1.38.  128^3, 60 views of 256^2 within 7 degrees: 456
+//    -> 375 us.
 constexpr int32_t kPlaneFwdBit = 64;
 constexpr double kPlaneFwdMinPitch = 0.75;
+constexpr double kPlaneFwdMinPitchLarge = 0.5;
+constexpr int64_t kPlaneLargeCube = 1 << 20;
 constexpr double kPlaneFwdMaxRatio = 0.02;
 constexpr int32_t kPlaneGeneralBit = 128;
 constexpr double kPlaneGeneralRatio = 0.035;
-// The thresholds above as walk rules (the default of every size bucket that
-// tomo_autotune or tomo_set_plane_rules has not set).
-inline tomo_plane_rules default_plane_rules()
+// The thresholds above as walk rules of a cube (the default of every size
+// bucket that tomo_autotune or tomo_set_plane_rules has not set).
+inline tomo_plane_rules default_plane_rules(const tomo_cube_geom &c)
 {
     tomo_plane_rules r;
     r.min_pitch = kPlaneMinPitch;
-    r.fwd_min_pitch = kPlaneFwdMinPitch;
+    r.fwd_min_pitch = (int64_t)c.nx * c.ny * c.nz >= kPlaneLargeCube
+                          ? kPlaneFwdMinPitchLarge : kPlaneFwdMinPitch;
     r.fwd_max_ratio = kPlaneFwdMaxRatio;
     r.general_ratio = kPlaneGeneralRatio;
     r.fwd_group = 0.0;

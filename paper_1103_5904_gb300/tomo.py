@@ -610,6 +610,9 @@ def tomo_set_plane_rules(rules=None, geom=None, nu=None, nv=None,
     if rules is not None:
         d = {"min_pitch": 0.16, "fwd_min_pitch": 0.75, "fwd_max_ratio": 0.02,
              "general_ratio": 0.035, "fwd_group": 0.0, "adj_group": 0.0}
+        if geom is not None and \
+                int(geom["nx"]) * int(geom["ny"]) * int(geom["nz"]) >= 1 << 20:
+            d["fwd_min_pitch"] = 0.5
         unknown = set(rules) - set(RULE_FIELDS)
         if unknown:
             raise ValueError("unknown rule(s) %s" % sorted(unknown))
