@@ -234,15 +234,7 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
         CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->setup_done, 0));
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->layout_used.p, 0, sizeof(unsigned), s));
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->per_ray_fwd.p, 0, sizeof(unsigned), s));
-        ctx->fwd_plane_possible = false;
-        ctx->fwd_plane_all = true;
-        ctx->plane_possible = false;
-        for (int32_t i = 0; i < g->n_img; ++i) {
-            const bool f = plane_forward_estimate(ptg[i], c, rules);
-            ctx->plane_possible |= plane_estimate(ptg[i], c, rules);
-            ctx->fwd_plane_possible |= f;
-            ctx->fwd_plane_all &= f;
-        }
+        estimate_walks(ctx, c, g, ptg, rules);
         LAUNCH(ctx, TOMO_K_SETUP, s,
                launch_frames((const tomo_pointing *)ctx->ptg.p, g->n_img, g->nu,
                              g->nv, n_frames, (Frame *)ctx->frames.p,
@@ -269,15 +261,7 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                                   cudaMemcpyHostToDevice, s));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->layout_used.p, 0, sizeof(unsigned), s));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->per_ray_fwd.p, 0, sizeof(unsigned), s));
-    ctx->fwd_plane_possible = false;
-    ctx->fwd_plane_all = true;
-    ctx->plane_possible = false;
-    for (size_t i = 0; i < n_img; ++i) {
-        const bool f = plane_forward_estimate(ptg[i], c, rules);
-        ctx->plane_possible |= plane_estimate(ptg[i], c, rules);
-        ctx->fwd_plane_possible |= f;
-        ctx->fwd_plane_all &= f;
-    }
+    estimate_walks(ctx, c, g, ptg, rules);
     LAUNCH(ctx, TOMO_K_SETUP, s,
            launch_frames((const tomo_pointing *)ctx->ptg.p, g->n_img, g->nu,
                          g->nv, n_frames, (Frame *)ctx->frames.p,
@@ -362,6 +346,74 @@ bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
     const double dmin = fmin(c->dx, fmin(c->dy, c->dz));
     const double pitch = p.d_obs * fabs(tan(p.cdelt_u)) / dmin;
     return pitch >= 0.9 * r.fwd_min_pitch || lo < 1.5 * r.fwd_max_ratio;
+}
+
+HintGuess guess_hint(const tomo_pointing &p, const tomo_cube_geom *c,
+                     const tomo_image_geom *g, const tomo_plane_rules &r)
+{
+    // k_frames' frame and plane_hint in the same formulas; comparisons closer
+    // than kNear (relative to unit vectors and thresholds) count as open
+    constexpr double kNear = 1e-9;
+    const double cl = cos(p.lat), sl = sin(p.lat);
+    const double co = cos(p.lon), so = sin(p.lon);
+    const double w[3] = { -cl * co, -cl * so, -sl };
+    const double n1 = sqrt(w[0] * w[0] + w[1] * w[1]);
+    const double a1[3] = { w[1] / n1, -w[0] / n1, 0.0 };
+    const double a2[3] = { a1[1] * w[2], -a1[0] * w[2],
+                           a1[0] * w[1] - a1[1] * w[0] };
+    const double cr = cos(p.roll), sr = sin(p.roll);
+    const double tu = tan((0.5 * (g->nu - 1) - p.crpix_u) * p.cdelt_u + p.crval_u);
+    const double tv = tan((0.5 * (g->nv - 1) - p.crpix_v) * p.cdelt_v + p.crval_v);
+    const double vox[3] = { c->dx, c->dy, c->dz };
+    double e1[3], u[3];
+    for (int a = 0; a < 3; ++a) {
+        e1[a] = cr * a1[a] + sr * a2[a];
+        u[a] = w[a] + tu * e1[a] + tv * (-sr * a1[a] + cr * a2[a]);
+    }
+    const double most = fmax(fabs(u[0]), fmax(fabs(u[1]), fabs(u[2])));
+    const double step = p.d_obs * fabs(tan(p.cdelt_u));
+    HintGuess h = { 0u, false, true };
+    for (int M = 0; M < 3; ++M) {
+        if (fabs(u[M]) < most * (1.0 - kNear)) continue;
+        double lat[3], best = 0.0, lo = INFINITY;
+        for (int a = 0; a < 3; ++a) {
+            if (a == M) continue;
+            lat[a] = fabs(e1[a] - u[a] * e1[M] / u[M]);
+            best = fmax(best, lat[a]);
+            lo = fmin(lo, fabs(u[a]) / fabs(u[M]));
+        }
+        for (int L = 0; L < 3; ++L) {
+            if (L == M || lat[L] < best - kNear) continue;
+            const double pitch = step / vox[L];
+            const bool may = pitch >= r.min_pitch * (1.0 - kNear);
+            const bool sure = pitch >= r.min_pitch * (1.0 + kNear);
+            if (may) h.layouts |= 1u << L;
+            h.fwd_may |= may && (pitch >= r.fwd_min_pitch * (1.0 - kNear) ||
+                                 lo < r.fwd_max_ratio + kNear);
+            h.fwd_sure &= sure && (pitch >= r.fwd_min_pitch * (1.0 + kNear) ||
+                                   lo < r.fwd_max_ratio - kNear);
+        }
+    }
+    return h;
+}
+
+void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
+                    const tomo_image_geom *g, const tomo_pointing *ptg,
+                    const tomo_plane_rules &rules)
+{
+    ctx->fwd_plane_possible = ctx->plane_possible = false;
+    ctx->fwd_plane_all = ctx->fwd_plane_sure = true;
+    ctx->lay_adj = ctx->lay_fwd = 0u;
+    for (int32_t i = 0; i < g->n_img; ++i) {
+        const bool f = plane_forward_estimate(ptg[i], c, rules);
+        ctx->plane_possible |= plane_estimate(ptg[i], c, rules);
+        ctx->fwd_plane_possible |= f;
+        ctx->fwd_plane_all &= f;
+        const HintGuess h = guess_hint(ptg[i], c, g, rules);
+        ctx->lay_adj |= h.layouts;
+        if (h.fwd_may) ctx->lay_fwd |= h.layouts;
+        ctx->fwd_plane_sure &= h.fwd_sure;
+    }
 }
 
 bool use_plane(const tomo_ctx *ctx, const tomo_cube_geom *c, Tiling t,
@@ -461,14 +513,16 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
         tomo_status st;
         if ((st = ensure_pairs(ctx, c, n_frames))) return st;
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
+        const unsigned lays = all ? ctx->lay_adj : ctx->lay_fwd;
         for (int L = 0; L <= 2; ++L)
-            LAUNCH(ctx, TOMO_K_LAYOUT, s,
+            if ((lays >> L) & 1u)
+                LAUNCH(ctx, TOMO_K_LAYOUT, s,
                    launch_to_pairs(cube_dev, dtype, ctx->pr[L].p, L, c,
                                    n_frames, used,
                                    all ? 1u << L : 1u << (8 + L), done,
                                    ctx->num_sms, s));
         PlaneCubes pc = { { ctx->pr[0].p, ctx->pr[1].p, ctx->pr[2].p } };
-        if (!all)
+        if (!all && !ctx->fwd_plane_sure)
             LAUNCH(ctx, TOMO_K_FORWARD, s,
                    launch_forward(rays, prm, cube_dev, dtype, fstride, true,
                                   mask, out, g->n_img, g->nu, g->nv, c->nx,
@@ -484,13 +538,15 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
     }
     if (use_plane(ctx, c, t, true) && (all || ctx->fwd_plane_possible)) {
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
+        const unsigned lays = all ? ctx->lay_adj : ctx->lay_fwd;
         for (int L = 1; L <= 2; ++L)
-            LAUNCH(ctx, TOMO_K_LAYOUT, s,
+            if ((lays >> L) & 1u)
+                LAUNCH(ctx, TOMO_K_LAYOUT, s,
                    launch_to_layout(cube_dev, dtype, L == 1 ? ctx->lay1.p : ctx->lay2.p,
                                     L, c, n_frames, used,
                                     all ? 1u << L : 1u << (8 + L), done, s));
         PlaneCubes pc = { { cube_dev, ctx->lay1.p, ctx->lay2.p } };
-        if (!all)
+        if (!all && !ctx->fwd_plane_sure)
             LAUNCH(ctx, TOMO_K_FORWARD, s,
                    launch_forward(rays, prm, cube_dev, dtype, fstride,
                                   n_frames > 1, mask, out, g->n_img, g->nu,
@@ -529,7 +585,8 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
         const int64_t fstride = (int64_t)c->nx * c->ny * c->nz;
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
         for (int L = 0; L <= 2; ++L)
-            LAUNCH(ctx, TOMO_K_LAYOUT, s,
+            if ((ctx->lay_adj >> L) & 1u)
+                LAUNCH(ctx, TOMO_K_LAYOUT, s,
                    launch_zero_layout((float *)ctx->pr[L].p, L,
                                       2 * fstride * (n_frames - 1), used,
                                       done, ctx->num_sms, s));
@@ -542,7 +599,8 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
                    plane_group(ctx, c, g, true, 8 * fstride * (n_frames - 1),
                                n_frames - 1)));
         for (int L = 0; L <= 2; ++L)
-            LAUNCH(ctx, TOMO_K_LAYOUT, s,
+            if ((ctx->lay_adj >> L) & 1u)
+                LAUNCH(ctx, TOMO_K_LAYOUT, s,
                    launch_add_pairs(ctx->pr[L].p, cube, L, c, n_frames, used,
                                     done, ctx->num_sms, s));
         return TOMO_OK;
@@ -550,24 +608,24 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
     if (use_plane(ctx, c, t, false) && ctx->plane_possible) {
         const int64_t fstride = (int64_t)c->nx * c->ny * c->nz;
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
-        float *a1 = (float *)ctx->lay1.p, *a2 = (float *)ctx->lay2.p;
-        LAUNCH(ctx, TOMO_K_LAYOUT, s,
-               launch_zero_layout(a1, 1, fstride * n_frames, used, done,
-                                  ctx->num_sms, s));
-        LAUNCH(ctx, TOMO_K_LAYOUT, s,
-               launch_zero_layout(a2, 2, fstride * n_frames, used, done,
-                                  ctx->num_sms, s));
-        PlaneAcc pa = { { cube, a1, a2 } };
+        float *a[3] = { cube, (float *)ctx->lay1.p, (float *)ctx->lay2.p };
+        for (int L = 1; L <= 2; ++L)
+            if ((ctx->lay_adj >> L) & 1u)
+                LAUNCH(ctx, TOMO_K_LAYOUT, s,
+                       launch_zero_layout(a[L], L, fstride * n_frames, used,
+                                          done, ctx->num_sms, s));
+        PlaneAcc pa = { { a[0], a[1], a[2] } };
         LAUNCH(ctx, TOMO_K_ADJOINT, s,
                launch_adjoint_plane(
                    rays, prm, images, mask, pa, fstride, n_frames > 1,
                    g->n_img, g->nu, g->nv, c, done, s,
                    plane_group(ctx, c, g, true, 4 * fstride * n_frames,
                                n_frames)));
-        LAUNCH(ctx, TOMO_K_LAYOUT, s,
-               launch_add_from_layout(a1, cube, 1, c, n_frames, used, done, s));
-        LAUNCH(ctx, TOMO_K_LAYOUT, s,
-               launch_add_from_layout(a2, cube, 2, c, n_frames, used, done, s));
+        for (int L = 1; L <= 2; ++L)
+            if ((ctx->lay_adj >> L) & 1u)
+                LAUNCH(ctx, TOMO_K_LAYOUT, s,
+                       launch_add_from_layout(a[L], cube, L, c, n_frames, used,
+                                              done, s));
         return TOMO_OK;
     }
     const int64_t fstride = (int64_t)c->nx * c->ny * c->nz;
@@ -629,8 +687,10 @@ tomo_status op_forward(tomo_ctx *ctx, const void *src, tomo_dtype dtype,
                            (all || ctx->fwd_plane_possible);
         if (plane) {
             const unsigned *used = (const unsigned *)ctx->layout_used.p;
+            const unsigned lays = all ? ctx->lay_adj : ctx->lay_fwd;
             for (int L = 1; L <= 2; ++L)
-                LAUNCH(ctx, TOMO_K_LAYOUT, s,
+                if ((lays >> L) & 1u)
+                    LAUNCH(ctx, TOMO_K_LAYOUT, s,
                        launch_b_to_layout(ctx->pr[0].p, ctx->pr[L].p, L, c,
                                           used, all ? 1u << L : 1u << (8 + L),
                                           done, s));
@@ -697,7 +757,8 @@ tomo_status op_adjoint(tomo_ctx *ctx, const float *images, const uint8_t *mask,
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->pr[0].p, 0, 8 * (size_t)n, s));
         if (plane)
             for (int L = 1; L <= 2; ++L)
-                LAUNCH(ctx, TOMO_K_LAYOUT, s,
+                if ((ctx->lay_adj >> L) & 1u)
+                    LAUNCH(ctx, TOMO_K_LAYOUT, s,
                        launch_zero_layout((float *)ctx->pr[L].p, L, 2 * n,
                                           used, done, ctx->num_sms, s));
         PlaneAcc pa = { { (float *)ctx->pr[0].p, (float *)ctx->pr[1].p,
@@ -710,7 +771,8 @@ tomo_status op_adjoint(tomo_ctx *ctx, const float *images, const uint8_t *mask,
                                 plane_group(ctx, c, g, true, 8 * n, 1)));
         if (plane)
             for (int L = 1; L <= 2; ++L)
-                LAUNCH(ctx, TOMO_K_LAYOUT, s,
+                if ((ctx->lay_adj >> L) & 1u)
+                    LAUNCH(ctx, TOMO_K_LAYOUT, s,
                        launch_add_b_layout(ctx->pr[L].p, ctx->pr[0].p, L, c,
                                            used, done, s));
         LAUNCH(ctx, TOMO_K_VECTOR, s,

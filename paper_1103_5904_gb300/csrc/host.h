@@ -78,6 +78,13 @@ struct tomo_ctx {
     // some image of the cached geometry may have a valid plane hint (the
     // same kind of estimate; when false the per-ray transpose runs)
     bool plane_possible = true;
+    // layouts (bit L) that some image of the cached geometry may walk in: in
+    // P^T (or with every image plane by plane), and in the plane forward;
+    // layout passes of the others are not launched
+    unsigned lay_adj = 7u, lay_fwd = 7u;
+    // every image of the cached geometry certainly selects the plane forward:
+    // no per-ray forward is launched
+    bool fwd_plane_sure = false;
     // cube copies (forward) / accumulators (transpose) in layouts 1 and 2
     tomo::host::DevBuf lay1, lay2;
     // two-value buffers (8 bytes per voxel) in layouts 0, 1, 2: frame pairs
@@ -165,6 +172,20 @@ bool plane_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                     const tomo_plane_rules &r);
 bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                             const tomo_plane_rules &r);
+// What the device's plane_hint (setup.cu) gives for an image, evaluated on the
+// host with a margin far above rounding: the layouts it may name if the hint
+// may be valid (0: certainly not valid), whether it may and whether it
+// certainly selects the plane forward.
+struct HintGuess {
+    unsigned layouts;
+    bool fwd_may, fwd_sure;
+};
+HintGuess guess_hint(const tomo_pointing &p, const tomo_cube_geom *c,
+                     const tomo_image_geom *g, const tomo_plane_rules &r);
+// Fills the context's per-geometry schedule estimates.
+void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
+                    const tomo_image_geom *g, const tomo_pointing *ptg,
+                    const tomo_plane_rules &rules);
 tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          int32_t n_frames, const tomo_image_geom *g,
                          const tomo_pointing *ptg, cudaStream_t s);
