@@ -456,13 +456,13 @@ k_vec_batched(const VecDesc *__restrict__ descs,
 #pragma unroll
                 for (int k = 0; k < kVecUnroll; ++k) a0.add_prod(u[k], v[k]);
             } else if constexpr (kOp == V_UPDATE) {
-                const float alpha = (float)d.S[S_ALPHA];
+                const StepF2 alpha(d.S[S_ALPHA]), minus(-d.S[S_ALPHA]);
                 float x[kVecUnroll] = {}, r[kVecUnroll] = {}, b[kVecUnroll] = {};
                 vec_group(c0, c1, g, [&](int64_t i, int k) {
-                    x[k] = fmaf(alpha, d.p[i], d.x[i]);
+                    x[k] = axpy(alpha, d.p[i], d.x[i]);
                     r[k] = (d.mm != nullptr && d.mm[i] != 0)
                                ? 0.0f
-                               : fmaf(-alpha, d.q[i], d.r[i]);
+                               : axpy(minus, d.q[i], d.r[i]);
                     b[k] = d.b[i];
                 });
                 vec_group(c0, c1, g, [&](int64_t i, int k) {
@@ -472,10 +472,10 @@ k_vec_batched(const VecDesc *__restrict__ descs,
                     a1.add_prod_sum(x[k], r[k], b[k]);
                 });
             } else if constexpr (kOp == V_DIR) {
-                const float beta = (float)d.S[S_BETA];
+                const StepF2 beta(d.S[S_BETA]);
                 float v[kVecUnroll] = {};
                 vec_group(c0, c1, g, [&](int64_t i, int k) {
-                    v[k] = fmaf(beta, d.p[i], d.r[i]);
+                    v[k] = axpy(beta, d.p[i], d.r[i]);
                 });
                 vec_group(c0, c1, g, [&](int64_t i, int k) { d.p[i] = v[k]; });
             }

@@ -59,6 +59,36 @@ struct SumF2 {
     }
 };
 
+// A CG scalar (alpha or beta) as a pair of floats, hi + lo, good to 2^-48.
+// Rounded to one float, its relative error of up to 2^-24 is the same in every
+// element: an error along p as a whole, not noise that averages out over the
+// voxels.  CG amplifies it once a Ritz value has converged on the largest
+// eigenvalue, and which float alpha rounds to changes with the order of the
+// transpose's float additions: x of 20 iterations (128^3, 60 views of 256^2)
+// was 6e-6 to 3e-4 off its 64-bit value and two runs differed by up to 5e-4;
+// with the pair 6e-6 to 2e-5 and 4e-6 to 2e-5.  The passes that use it are
+// bound by memory.
+struct StepF2 {
+    float hi, lo;
+    __device__ __forceinline__ explicit StepF2(double v)
+        : hi((float)v), lo((float)(v - (double)(float)v)) {}
+};
+
+// x + a v, rounded once but for terms of order 2^-48: the product and the sum
+// are split exactly (TwoProduct, TwoSum).  Where these give NaN (overflow,
+// non-finite operands) the plain multiply-add's value stands.
+__device__ __forceinline__ float axpy(const StepF2 &a, float v, float x)
+{
+    const float p = __fmul_rn(a.hi, v);
+    const float e = fmaf(a.lo, v, fmaf(a.hi, v, -p));
+    const float s = __fadd_rn(x, p);
+    const float bb = __fsub_rn(s, x);
+    const float es = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)),
+                               __fsub_rn(p, bb));
+    const float y = __fadd_rn(s, __fadd_rn(es, e));
+    return y == y ? y : fmaf(a.hi, v, x);
+}
+
 __device__ __forceinline__ double warp_sum(double v)
 {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);

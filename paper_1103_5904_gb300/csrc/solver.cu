@@ -218,12 +218,12 @@ __global__ void k_cg_pq(const float *__restrict__ p, const float *__restrict__ q
 struct CgUpdateElem {
     float *x, *r;
     const float *p, *q, *b;
-    float alpha;
+    StepF2 alpha, minus;  // alpha and -alpha
     __device__ __forceinline__ void operator()(int64_t i, bool out,
                                                SumF2 v[2]) const
     {
-        const float xi = fmaf(alpha, p[i], x[i]);
-        const float ri = out ? 0.0f : fmaf(-alpha, q[i], r[i]);
+        const float xi = axpy(alpha, p[i], x[i]);
+        const float ri = out ? 0.0f : axpy(minus, q[i], r[i]);
         x[i] = xi;
         r[i] = ri;
         v[0].add_prod(ri, ri);
@@ -241,7 +241,8 @@ __global__ void k_cg_update(float *__restrict__ x, float *__restrict__ r,
 {
     if (S[S_DONE] != 0.0) return;
     SumF2 a[2];
-    const CgUpdateElem f = { x, r, p, q, b, (float)S[S_ALPHA] };
+    const CgUpdateElem f = { x, r, p, q, b, StepF2(S[S_ALPHA]),
+                             StepF2(-S[S_ALPHA]) };
     masked_elements(mm, mm_n, n, f, a);
     double v[2] = { a[0].value(), a[1].value() };
     double tot[2];
@@ -254,10 +255,10 @@ __global__ void k_cg_direction(const float *__restrict__ r, float *p,
                                const double *__restrict__ S)
 {
     if (S[S_DONE] != 0.0) return;
-    const float beta = (float)S[S_BETA];
+    const StepF2 beta(S[S_BETA]);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        p[i] = direction_store(fmaf(beta, p[i], r[i]), p16, i);
+        p[i] = direction_store(axpy(beta, p[i], r[i]), p16, i);
     }
 }
 
