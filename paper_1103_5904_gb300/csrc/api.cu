@@ -10,6 +10,7 @@
 
 #include <cuda_runtime.h>
 
+#include "hint.cuh"
 #include "host.h"
 
 using namespace tomo;
@@ -231,6 +232,8 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
             return TOMO_OK;
         }
         // same rays, other walk rules: only the per-image hints change
+        // (the cache is invalid until the new hints and estimates are in)
+        ctx->key_valid = false;
         CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->setup_done, 0));
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->layout_used.p, 0, sizeof(unsigned), s));
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->per_ray_fwd.p, 0, sizeof(unsigned), s));
@@ -245,6 +248,7 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                              (unsigned *)ctx->per_ray_fwd.p, rules, s));
         CUDA_TRY(ctx, cudaEventRecord(ctx->setup_done, s));
         ctx->hint_key = hh;
+        ctx->key_valid = true;
         return TOMO_OK;
     }
     ctx->key_valid = false;
@@ -325,7 +329,7 @@ tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
     return ctx->rules_set ? ctx->rules : default_plane_rules(*c);
 }
 
-// The device's rules (setup.cu) evaluated from the boresight, with margins
+// The device's rules (hint.cuh) evaluated from the boresight, with margins
 // towards "may"; the pixel pitch with the smallest voxel side.
 bool plane_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                     const tomo_plane_rules &r)
@@ -348,54 +352,9 @@ bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
     return pitch >= 0.9 * r.fwd_min_pitch || lo < 1.5 * r.fwd_max_ratio;
 }
 
-HintGuess guess_hint(const tomo_pointing &p, const tomo_cube_geom *c,
-                     const tomo_image_geom *g, const tomo_plane_rules &r)
-{
-    // k_frames' frame and plane_hint in the same formulas; comparisons closer
-    // than kNear (relative to unit vectors and thresholds) count as open
-    constexpr double kNear = 1e-9;
-    const double cl = cos(p.lat), sl = sin(p.lat);
-    const double co = cos(p.lon), so = sin(p.lon);
-    const double w[3] = { -cl * co, -cl * so, -sl };
-    const double n1 = sqrt(w[0] * w[0] + w[1] * w[1]);
-    const double a1[3] = { w[1] / n1, -w[0] / n1, 0.0 };
-    const double a2[3] = { a1[1] * w[2], -a1[0] * w[2],
-                           a1[0] * w[1] - a1[1] * w[0] };
-    const double cr = cos(p.roll), sr = sin(p.roll);
-    const double tu = tan((0.5 * (g->nu - 1) - p.crpix_u) * p.cdelt_u + p.crval_u);
-    const double tv = tan((0.5 * (g->nv - 1) - p.crpix_v) * p.cdelt_v + p.crval_v);
-    const double vox[3] = { c->dx, c->dy, c->dz };
-    double e1[3], u[3];
-    for (int a = 0; a < 3; ++a) {
-        e1[a] = cr * a1[a] + sr * a2[a];
-        u[a] = w[a] + tu * e1[a] + tv * (-sr * a1[a] + cr * a2[a]);
-    }
-    const double most = fmax(fabs(u[0]), fmax(fabs(u[1]), fabs(u[2])));
-    const double step = p.d_obs * fabs(tan(p.cdelt_u));
-    HintGuess h = { 0u, false, true };
-    for (int M = 0; M < 3; ++M) {
-        if (fabs(u[M]) < most * (1.0 - kNear)) continue;
-        double lat[3], best = 0.0, lo = INFINITY;
-        for (int a = 0; a < 3; ++a) {
-            if (a == M) continue;
-            lat[a] = fabs(e1[a] - u[a] * e1[M] / u[M]);
-            best = fmax(best, lat[a]);
-            lo = fmin(lo, fabs(u[a]) / fabs(u[M]));
-        }
-        for (int L = 0; L < 3; ++L) {
-            if (L == M || lat[L] < best - kNear) continue;
-            const double pitch = step / vox[L];
-            const bool may = pitch >= r.min_pitch * (1.0 - kNear);
-            const bool sure = pitch >= r.min_pitch * (1.0 + kNear);
-            if (may) h.layouts |= 1u << L;
-            h.fwd_may |= may && (pitch >= r.fwd_min_pitch * (1.0 - kNear) ||
-                                 lo < r.fwd_max_ratio + kNear);
-            h.fwd_sure &= sure && (pitch >= r.fwd_min_pitch * (1.0 + kNear) ||
-                                   lo < r.fwd_max_ratio - kNear);
-        }
-    }
-    return h;
-}
+// Far above the rounding of the host's and the device's sines and products
+// (1e-15), far below any difference that matters for speed.
+constexpr double kHintTol = 1e-9;
 
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
@@ -409,7 +368,9 @@ void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
         ctx->plane_possible |= plane_estimate(ptg[i], c, rules);
         ctx->fwd_plane_possible |= f;
         ctx->fwd_plane_all &= f;
-        const HintGuess h = guess_hint(ptg[i], c, g, rules);
+        const PlaneHint h = plane_hint(ptg[i], image_frame(ptg[i]), g->nu, g->nv,
+                                       make_double3(c->dx, c->dy, c->dz), rules,
+                                       kHintTol);
         ctx->lay_adj |= h.layouts;
         if (h.fwd_may) ctx->lay_fwd |= h.layouts;
         ctx->fwd_plane_sure &= h.fwd_sure;

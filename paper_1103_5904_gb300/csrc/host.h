@@ -163,8 +163,7 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
                         const tomo_cube_geom *c, int32_t n_frames,
                         const tomo_image_geom *g, Tiling t,
                         const double *done, cudaStream_t s);
-// Builds (or reuses) the context's ray records for one geometry on `s`.
-// Host estimates of the device's per-image plane-walk rules (setup.cu) from
+// Host estimates of the device's per-image plane-walk rules (hint.cuh) from
 // the boresight: whether an image may get a valid hint, and whether it may
 // select the plane forward.  Only speed depends on them: the kernel that
 // runs when an estimate says no walks every ray per ray.
@@ -172,20 +171,13 @@ bool plane_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                     const tomo_plane_rules &r);
 bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                             const tomo_plane_rules &r);
-// What the device's plane_hint (setup.cu) gives for an image, evaluated on the
-// host with a margin far above rounding: the layouts it may name if the hint
-// may be valid (0: certainly not valid), whether it may and whether it
-// certainly selects the plane forward.
-struct HintGuess {
-    unsigned layouts;
-    bool fwd_may, fwd_sure;
-};
-HintGuess guess_hint(const tomo_pointing &p, const tomo_cube_geom *c,
-                     const tomo_image_geom *g, const tomo_plane_rules &r);
-// Fills the context's per-geometry schedule estimates.
+// Fills the context's per-geometry schedule: the estimates above and, from
+// plane_hint with a tolerance, the layouts whose passes are launched and
+// whether the per-ray forward is (results depend on these).
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules);
+// Builds (or reuses) the context's ray records for one geometry on `s`.
 tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          int32_t n_frames, const tomo_image_geom *g,
                          const tomo_pointing *ptg, cudaStream_t s);

@@ -13,58 +13,11 @@
 // e1 = unit(w x z), e2 = e1 x w, turned by the roll angle about w; gnomonic
 // (TAN) pixel angles theta = (i - crpix) cdelt + crval per axis; ray
 // direction unit(w + tan(theta_u) e1 + tan(theta_v) e2).
-#include <math.h>
-
-#include "tomo_internal.cuh"
+#include "hint.cuh"
 
 namespace tomo {
 
 namespace {
-
-// Hint for the plane-synchronous walk of one image: M = the axis along
-// which the line of sight of the image centre advances fastest, its
-// direction, and L = the axis (other than M) along which neighbouring pixels
-// of a row move at a fixed M plane.  Moving along the row turns the
-// direction by ~e1; at a fixed M plane the ray through u + e1 d is displaced
-// along e1 - u e1_M / u_M.  The hint is marked valid only when neighbouring
-// pixels are at least rules.min_pitch voxels of L apart at the distance of
-// Sun centre; the forward and walk-variant bits follow the other rules
-// (defaults: the measured thresholds in tomo_internal.cuh; tomo_autotune
-// can tune them per size bucket).  Only the walks' speed depends on the
-// hint.
-__device__ int32_t plane_hint(const tomo_pointing &p, const Frame &f, int nu,
-                              int nv, double3 vox, const tomo_plane_rules &rules)
-{
-    const double tu = tan((0.5 * (nu - 1) - p.crpix_u) * p.cdelt_u + p.crval_u);
-    const double tv = tan((0.5 * (nv - 1) - p.crpix_v) * p.cdelt_v + p.crval_v);
-    double u[3];
-    for (int a = 0; a < 3; ++a) u[a] = f.w[a] + tu * f.e1[a] + tv * f.e2[a];
-    int M = 0;
-    for (int a = 1; a < 3; ++a)
-        if (fabs(u[a]) > fabs(u[M])) M = a;
-    int L = -1;
-    double best = -1.0;
-    for (int a = 0; a < 3; ++a) {
-        if (a == M) continue;
-        const double lat = fabs(f.e1[a] - u[a] * f.e1[M] / u[M]);
-        if (lat > best) {
-            best = lat;
-            L = a;
-        }
-    }
-    const double dL = L == 0 ? vox.x : (L == 1 ? vox.y : vox.z);
-    const double pitch = p.d_obs * fabs(tan(p.cdelt_u)) / dL;
-    const bool valid = pitch >= rules.min_pitch;
-    double lo = INFINITY;  // the less steep minor component
-    for (int a = 0; a < 3; ++a)
-        if (a != M) lo = fmin(lo, fabs(u[a]));
-    lo /= fabs(u[M]);
-    const bool general = lo >= rules.general_ratio;
-    const bool fwd = valid && (pitch >= rules.fwd_min_pitch || lo < rules.fwd_max_ratio);
-    return (valid ? kPlaneHintValid : 0) | (fwd ? kPlaneFwdBit : 0) |
-           (general ? kPlaneGeneralBit : 0) | M | (L << 2) |
-           ((u[M] < 0.0) ? 16 : 0);
-}
 
 // One block per image: the FP64 frame, the image parameters and the tangent
 // tables tan(theta_u), tan(theta_v) (one value per column / row).
@@ -77,30 +30,11 @@ __global__ void k_frames(const tomo_pointing *__restrict__ ptg, int32_t nu,
     const int img = blockIdx.x;
     const tomo_pointing p = ptg[img];
     if (threadIdx.x == 0) {
-        Frame f;
-        const double cl = cos(p.lat), sl = sin(p.lat);
-        const double co = cos(p.lon), so = sin(p.lon);
-        f.o[0] = p.d_obs * cl * co;
-        f.o[1] = p.d_obs * cl * so;
-        f.o[2] = p.d_obs * sl;
-        f.w[0] = -cl * co;
-        f.w[1] = -cl * so;
-        f.w[2] = -sl;
-        // w x z = (w_y, -w_x, 0), of length cos(lat)
-        const double n1 = sqrt(f.w[0] * f.w[0] + f.w[1] * f.w[1]);
-        const double a1[3] = { f.w[1] / n1, -f.w[0] / n1, 0.0 };
-        const double a2[3] = { a1[1] * f.w[2] - a1[2] * f.w[1],
-                               a1[2] * f.w[0] - a1[0] * f.w[2],
-                               a1[0] * f.w[1] - a1[1] * f.w[0] };
-        const double cr = cos(p.roll), sr = sin(p.roll);
-        for (int a = 0; a < 3; ++a) {
-            f.e1[a] = cr * a1[a] + sr * a2[a];
-            f.e2[a] = -sr * a1[a] + cr * a2[a];
-        }
+        const Frame f = image_frame(p);
         frames[img] = f;
         ImgParam q;
         q.gain = (float)p.gain;
-        q.pad = plane_hint(p, f, nu, nv, vox, rules);
+        q.pad = plane_hint(p, f, nu, nv, vox, rules, 0.0).code;
         if (layout_used && (q.pad & kPlaneHintValid)) {
             // bit L: a plane transpose uses layout L; bit 8 + L: so does a
             // plane forward
