@@ -360,14 +360,10 @@ void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules)
 {
-    ctx->fwd_plane_possible = ctx->plane_possible = false;
     ctx->fwd_plane_all = ctx->fwd_plane_sure = true;
     ctx->lay_adj = ctx->lay_fwd = 0u;
     for (int32_t i = 0; i < g->n_img; ++i) {
-        const bool f = plane_forward_estimate(ptg[i], c, rules);
-        ctx->plane_possible |= plane_estimate(ptg[i], c, rules);
-        ctx->fwd_plane_possible |= f;
-        ctx->fwd_plane_all &= f;
+        ctx->fwd_plane_all &= plane_forward_estimate(ptg[i], c, rules);
         const PlaneHint h = plane_hint(ptg[i], image_frame(ptg[i]), g->nu, g->nv,
                                        make_double3(c->dx, c->dy, c->dz), rules,
                                        kHintTol);
@@ -468,7 +464,7 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
     // bit 1: every image plane-synchronous; else (bit 2) the images whose
     // hint marks the plane forward as faster, the rest per ray
     const bool all = (ctx->plane_sync & 2) != 0;
-    if (use_plane(ctx, c, t, true) && (all || ctx->fwd_plane_possible) &&
+    if (use_plane(ctx, c, t, true) && (all || ctx->lay_fwd != 0u) &&
         use_time_pairs(ctx, c, n_frames)) {
         // frame pairs side by side in every layout in use (layout 0 too)
         tomo_status st;
@@ -497,7 +493,7 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
                                n_frames - 1)));
         return TOMO_OK;
     }
-    if (use_plane(ctx, c, t, true) && (all || ctx->fwd_plane_possible)) {
+    if (use_plane(ctx, c, t, true) && (all || ctx->lay_fwd != 0u)) {
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
         const unsigned lays = all ? ctx->lay_adj : ctx->lay_fwd;
         for (int L = 1; L <= 2; ++L)
@@ -537,7 +533,7 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
 {
     const RayRec *rays = (const RayRec *)ctx->rays.p;
     const ImgParam *prm = (const ImgParam *)ctx->params.p;
-    if (use_plane(ctx, c, t, false) && ctx->plane_possible &&
+    if (use_plane(ctx, c, t, false) && ctx->lay_adj != 0u &&
         use_time_pairs(ctx, c, n_frames)) {
         // frame-pair accumulators in every layout in use, added into the
         // frames after the walk
@@ -566,7 +562,7 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
                                     done, ctx->num_sms, s));
         return TOMO_OK;
     }
-    if (use_plane(ctx, c, t, false) && ctx->plane_possible) {
+    if (use_plane(ctx, c, t, false) && ctx->lay_adj != 0u) {
         const int64_t fstride = (int64_t)c->nx * c->ny * c->nz;
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
         float *a[3] = { cube, (float *)ctx->lay1.p, (float *)ctx->lay2.p };
@@ -645,7 +641,7 @@ tomo_status op_forward(tomo_ctx *ctx, const void *src, tomo_dtype dtype,
         const bool all = (ctx->plane_sync & 2) != 0;
         const bool plane = use_plane(ctx, c, t, true) &&
                            plane_supported(c, 8) &&
-                           (all || ctx->fwd_plane_possible);
+                           (all || ctx->lay_fwd != 0u);
         if (plane) {
             const unsigned *used = (const unsigned *)ctx->layout_used.p;
             const unsigned lays = all ? ctx->lay_adj : ctx->lay_fwd;
@@ -713,7 +709,7 @@ tomo_status op_adjoint(tomo_ctx *ctx, const float *images, const uint8_t *mask,
         // dst += K (m' a - m b)
         if ((st = ensure_pairs(ctx, c, 1))) return st;
         const bool plane = use_plane(ctx, c, t, false) &&
-                           plane_supported(c, 8) && ctx->plane_possible;
+                           plane_supported(c, 8) && ctx->lay_adj != 0u;
         const unsigned *used = (const unsigned *)ctx->layout_used.p;
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->pr[0].p, 0, 8 * (size_t)n, s));
         if (plane)
@@ -930,12 +926,12 @@ tomo_status tomo_walk_plan(tomo_ctx *ctx, int32_t n_img, int32_t *codes_host)
                              cudaMemcpyDeviceToHost));
     // what the single-value walks of P and P^T run (Section 3.3.1): the
     // device hint, gated as the host gates the launches (option bits, the
-    // host estimates, the plane walk's buffer-size bound)
+    // layouts in use, the plane walk's buffer-size bound)
     const bool fits = plane_supported(&ctx->cached_cube, 4);
-    const bool adj_on = fits && (ctx->plane_sync & 1) && ctx->plane_possible;
+    const bool adj_on = fits && (ctx->plane_sync & 1) && ctx->lay_adj != 0u;
     const bool all = (ctx->plane_sync & 2) != 0;
     const bool fwd_on = fits && (ctx->plane_sync & (2 | 4)) &&
-                        (all || ctx->fwd_plane_possible);
+                        (all || ctx->lay_fwd != 0u);
     for (int32_t i = 0; i < n_img; ++i) {
         const int32_t h = prm[i].pad;
         const bool valid = (h & kPlaneHintValid) != 0;

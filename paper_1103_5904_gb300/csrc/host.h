@@ -69,18 +69,14 @@ struct tomo_ctx {
     // { count, image indices }: the images of the cached geometry whose hint
     // leaves them to the per-ray forward
     tomo::host::DevBuf per_ray_fwd;
-    // some image of the cached geometry may select the plane forward (a
-    // host-side upper bound of the device's per-image pixel-pitch test)
-    bool fwd_plane_possible = true;
-    // every image of the cached geometry may select the plane forward (the
-    // same estimate): the per-ray forward then runs in its listed form
+    // every image of the cached geometry lies above or near the threshold of
+    // the plane forward (a coarse host estimate): the per-ray forward then
+    // runs in its listed form
     bool fwd_plane_all = false;
-    // some image of the cached geometry may have a valid plane hint (the
-    // same kind of estimate; when false the per-ray transpose runs)
-    bool plane_possible = true;
     // layouts (bit L) that some image of the cached geometry may walk in: in
     // P^T (or with every image plane by plane), and in the plane forward;
-    // layout passes of the others are not launched
+    // layout passes of the others are not launched, and with no layout at all
+    // the per-ray kernels run alone
     unsigned lay_adj = 7u, lay_fwd = 7u;
     // every image of the cached geometry certainly selects the plane forward:
     // no per-ray forward is launched
@@ -163,17 +159,17 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
                         const tomo_cube_geom *c, int32_t n_frames,
                         const tomo_image_geom *g, Tiling t,
                         const double *done, cudaStream_t s);
-// Host estimates of the device's per-image plane-walk rules (hint.cuh) from
-// the boresight: whether an image may get a valid hint, and whether it may
-// select the plane forward.  Only speed depends on them: the kernel that
-// runs when an estimate says no walks every ray per ray.
+// Coarse host estimates, from the boresight and with wide margins, of whether
+// an image may get a valid hint and whether it lies above or near the
+// thresholds of the plane forward.  Only speed depends on them: they choose
+// between kernels that read the device's hints themselves.
 bool plane_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                     const tomo_plane_rules &r);
 bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
                             const tomo_plane_rules &r);
-// Fills the context's per-geometry schedule: the estimates above and, from
-// plane_hint with a tolerance, the layouts whose passes are launched and
-// whether the per-ray forward is (results depend on these).
+// Fills the context's per-geometry schedule: from plane_hint with a tolerance,
+// the layouts whose passes are launched and whether the per-ray forward is
+// (results depend on these); from the estimate above, its listed form.
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules);
