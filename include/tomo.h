@@ -141,10 +141,9 @@ typedef struct tomo_ctx tomo_ctx;
                                   on every image; bit 2 for P on the images
                                   where it measured faster: views within
                                   ~1 degree of a cube-axis plane, or pixels
-                                  at least 0.75 voxel apart (0.5 on cubes of
-                                  at least 2^20 voxels; per ray on the
-                                  others).  A set bit
-                                  makes the rays of a warp walk the cube one
+                                  at least 0.75 voxel apart (or less, see
+                                  fwd_min_pitch in tomo_plane_rules; per ray
+                                  on the others).  A set bit makes the rays of a warp walk the cube one
                                   plane of the image's major axis at a time,
                                   on a copy of the cube stored with the
                                   image's lateral axis fastest, so the voxels
@@ -393,9 +392,14 @@ typedef struct {
     double min_pitch;      /* plane-synchronous walks when pitch >= this,
                               per-ray walks below (default 0.16) */
     double fwd_min_pitch;  /* P plane-synchronous when pitch >= this ... */
-    double fwd_max_ratio;  /* ... or ratio < this (defaults 0.75, or 0.5
-                              for cubes of at least 2^20 voxels, and 0.02;
-                              P per ray otherwise) */
+    double fwd_max_ratio;  /* ... or ratio < this (P per ray otherwise;
+                              defaults 0.75 and 0.02; 0.5 in place of 0.75
+                              for cubes of at least 2^20 voxels in batched
+                              calls and for Thomson B in one walk, and in
+                              other single calls when it takes every image
+                              and the rows of nx voxels are a multiple of
+                              128 bytes long as stored or the walk is on
+                              frame pairs, TOMO_OPT_CHANNELS) */
     double general_ratio;  /* plane walks cross every slab with the general
                               three-segment body when ratio >= this, else
                               they count the slabs to the next crossing of

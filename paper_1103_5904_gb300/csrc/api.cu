@@ -206,11 +206,71 @@ CubeDev cube_dev(const tomo_cube_geom *c)
     return d;
 }
 
+bool use_time_pairs(const tomo_ctx *ctx, const tomo_cube_geom *c,
+                    int32_t n_frames)
+{
+    return n_frames > 1 && (ctx->channels & 1) && plane_supported(c, 8);
+}
+
+// Thomson B in one walk on two values per voxel.
+static bool use_one_b(const tomo_ctx *ctx, const tomo_image_geom *g,
+                      int32_t n_frames)
+{
+    return g->kind == TOMO_KIND_B && n_frames == 1 && (ctx->channels & 2);
+}
+
+// Far above the rounding of the host's and the device's sines and products
+// (1e-15), far below any difference that matters for speed.
+constexpr double kHintTol = 1e-9;
+
+// The row that P gathers from, as default_plane_rules takes it.
+static int64_t forward_row(const tomo_ctx *ctx, const tomo_cube_geom *c,
+                           int32_t n_frames, const tomo_image_geom *g,
+                           tomo_dtype dtype)
+{
+    if (n_frames > 1) return use_time_pairs(ctx, c, n_frames) ? kAnyRow : kTimeRow;
+    if (use_one_b(ctx, g, n_frames)) return kAnyRow;
+    // the Thomson prologue writes floats
+    const bool bf16 = dtype == TOMO_BF16 && g->kind == TOMO_KIND_EMISSION;
+    return (int64_t)c->nx * (bf16 ? 2 : 4);
+}
+
+// The walk rules of a stack of images (geom: hash of its geometry).  Where the
+// defaults would let a stack's images through from kPlaneFwdMinPitchLarge on,
+// they do so only when that takes every image: a stack split between the two
+// forwards pays for both launches' tails and the layout copies, which the gain
+// on half of its images does not cover (17 views of 384^2, 192 x 163 x 169
+// cube, pixels 0.53 voxel of x and 0.45 of y apart: 0.52 ms split, 0.47 per
+// ray; three frames 181 x 154 x 198: 0.75 against 0.67 ms).  Thomson B walks
+// both kinds of image in one launch (one_walk): 0.52 ms split, 0.64 per ray on
+// 128 x 93 x 116.
+static tomo_plane_rules stack_rules(tomo_ctx *ctx, const tomo_cube_geom *c,
+                                    const tomo_image_geom *g,
+                                    const tomo_pointing *ptg, int64_t row,
+                                    bool one_walk, uint64_t geom)
+{
+    bool built_in;
+    tomo_plane_rules r = rules_for(ctx, c, g, row, &built_in);
+    if (!built_in || one_walk || r.fwd_min_pitch != kPlaneFwdMinPitchLarge) return r;
+    if (!ctx->dense_valid || ctx->dense_key != geom) {
+        ctx->dense = true;
+        for (int32_t i = 0; i < g->n_img && ctx->dense; ++i)
+            ctx->dense = plane_hint(ptg[i], image_frame(ptg[i]), g->nu, g->nv,
+                                    make_double3(c->dx, c->dy, c->dz), r,
+                                    kHintTol).fwd_sure;
+        ctx->dense_key = geom;
+        ctx->dense_valid = true;
+    }
+    if (!ctx->dense) r.fwd_min_pitch = kPlaneFwdMinPitch;
+    return r;
+}
+
 // Builds (or reuses) the ray records and image parameters of a geometry on
 // `s`.  On return, work on `s` is ordered after the records are complete.
 tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          int32_t n_frames, const tomo_image_geom *g,
-                         const tomo_pointing *ptg, cudaStream_t s)
+                         const tomo_pointing *ptg, tomo_dtype dtype,
+                         cudaStream_t s)
 {
     uint64_t h = 1469598103934665603ull;
     const int32_t cn[4] = { c->nx, c->ny, c->nz, n_frames };
@@ -219,7 +279,9 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
     h = fnv1a(h, cv, sizeof(cv));
     h = fnv1a(h, g, sizeof(*g));
     h = fnv1a(h, ptg, sizeof(tomo_pointing) * (size_t)g->n_img);
-    const tomo_plane_rules rules = rules_for(ctx, c, g);
+    const tomo_plane_rules rules =
+        stack_rules(ctx, c, g, ptg, forward_row(ctx, c, n_frames, g, dtype),
+                    use_one_b(ctx, g, n_frames), h);
     const uint64_t hh = fnv1a(h, &rules, sizeof(rules));
     tomo_status st;
     if ((st = ensure(ctx, ctx->layout_used, sizeof(unsigned))) ||
@@ -320,13 +382,16 @@ Tiling tiling_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
 }
 
 tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
-                           const tomo_image_geom *g)
+                           const tomo_image_geom *g, int64_t row, bool *built_in)
 {
+    if (built_in) *built_in = false;
     for (const Tuned &t : ctx->tuned)
         if (t.nx == c->nx && t.ny == c->ny && t.nz == c->nz && t.nu == g->nu &&
             t.nv == g->nv)
             return t.rules;
-    return ctx->rules_set ? ctx->rules : default_plane_rules(*c);
+    if (ctx->rules_set) return ctx->rules;
+    if (built_in) *built_in = true;
+    return default_plane_rules(*c, row);
 }
 
 // The device's rules (hint.cuh) evaluated from the boresight, with margins
@@ -351,10 +416,6 @@ bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
     const double pitch = p.d_obs * fabs(tan(p.cdelt_u)) / dmin;
     return pitch >= 0.9 * r.fwd_min_pitch || lo < 1.5 * r.fwd_max_ratio;
 }
-
-// Far above the rounding of the host's and the device's sines and products
-// (1e-15), far below any difference that matters for speed.
-constexpr double kHintTol = 1e-9;
 
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
@@ -437,12 +498,6 @@ int plane_group(const tomo_ctx *ctx, const tomo_cube_geom *c,
     if (!adjoint) return walked_bytes >= l2 / 4 ? n_img : 1;
     if (walked_bytes <= 2 * l2) return 1;
     return n_acc > 1 ? n_img : 8;
-}
-
-bool use_time_pairs(const tomo_ctx *ctx, const tomo_cube_geom *c,
-                    int32_t n_frames)
-{
-    return n_frames > 1 && (ctx->channels & 1) && plane_supported(c, 8);
 }
 
 // The per-ray forward's image list when the host estimate says every image
@@ -632,7 +687,7 @@ tomo_status op_forward(tomo_ctx *ctx, const void *src, tomo_dtype dtype,
     const float2 *mf = (const float2 *)ctx->thf.p;
     const float *rho2 = (const float *)ctx->rho2.p;
     const bool bf16 = dtype == TOMO_BF16;
-    if (g->kind == TOMO_KIND_B && n_frames == 1 && (ctx->channels & 2)) {
+    if (use_one_b(ctx, g, n_frames)) {
         // one walk on (m' K x, m K x) pairs: y = g s' - rho^2 g s
         if ((st = ensure_pairs(ctx, c, 1))) return st;
         LAUNCH(ctx, TOMO_K_VECTOR, s,
@@ -704,7 +759,7 @@ tomo_status op_adjoint(tomo_ctx *ctx, const float *images, const uint8_t *mask,
     tomo_status st;
     const float2 *mf = (const float2 *)ctx->thf.p;
     const float *rho2 = (const float *)ctx->rho2.p;
-    if (b && n_frames == 1 && (ctx->channels & 2)) {
+    if (use_one_b(ctx, g, n_frames)) {
         // one walk scattering (g y, rho^2 g y) into pair accumulators, then
         // dst += K (m' a - m b)
         if ((st = ensure_pairs(ctx, c, 1))) return st;
@@ -1007,7 +1062,7 @@ tomo_status tomo_project(tomo_ctx *ctx, const tomo_cube_geom *cube,
     cudaStream_t s = (cudaStream_t)stream;
     const Tiling tl = tiling_for(ctx, cube, img);
     if ((st = ensure_plane(ctx, cube, n_frames, tl)) ||
-        (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, s)))
+        (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, dtype, s)))
         return st;
     if (img->kind != TOMO_KIND_EMISSION) {
         // the Thomson prologue applies the map mask with M or M'
@@ -1058,7 +1113,7 @@ tomo_status tomo_backproject(tomo_ctx *ctx, const tomo_cube_geom *cube,
     if (img->n_img == 0) return TOMO_OK;
     const Tiling tl = tiling_for(ctx, cube, img);
     if ((st = ensure_plane(ctx, cube, n_frames, tl)) ||
-        (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, s)))
+        (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, TOMO_F32, s)))
         return st;
     if (img->kind != TOMO_KIND_EMISSION) {
         // dst += K T^T y: the Thomson epilogue skips the excluded voxels
@@ -1132,7 +1187,7 @@ tomo_status tomo_count_segments(tomo_ctx *ctx, const tomo_cube_geom *cube,
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return fail(ctx, TOMO_ERR_CUDA, "cannot select device");
     cudaStream_t s = (cudaStream_t)stream;
-    if ((st = prepare_rays(ctx, cube, 1, img, pointing_host, s))) return st;
+    if ((st = prepare_rays(ctx, cube, 1, img, pointing_host, TOMO_F32, s))) return st;
     if ((st = ensure(ctx, ctx->count64, sizeof(unsigned long long)))) return st;
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->count64.p, 0, sizeof(unsigned long long), s));
     LAUNCH(ctx, TOMO_K_FORWARD, s, launch_count((const RayRec *)ctx->rays.p, mask_dev, img->n_img,
@@ -1199,7 +1254,8 @@ tomo_status tomo_solve(tomo_ctx *ctx, const tomo_cube_geom *cube,
     const Tiling tl = tiling_for(ctx, cube, img);
     if (img->n_img > 0 &&
         ((st = ensure_plane(ctx, cube, n_frames, tl)) ||
-         (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, s)) ||
+         (st = prepare_rays(ctx, cube, n_frames, img, pointing_host,
+                            bf16 ? TOMO_BF16 : TOMO_F32, s)) ||
          (img->kind != TOMO_KIND_EMISSION &&
           (st = ensure_thomson(ctx, cube, img->limb_u, s)))))
         return st;

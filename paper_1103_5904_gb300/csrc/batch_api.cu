@@ -593,7 +593,8 @@ tomo_status time_schedule(tomo_ctx *ctx, const tomo_problem *p, Tiling t,
                           float *fwd_ms, float *adj_ms)
 {
     tomo_status st;
-    if ((st = prepare_rays(ctx, &p->cube, 1, &p->img, p->pointing_host, s)))
+    if ((st = prepare_rays(ctx, &p->cube, 1, &p->img, p->pointing_host,
+                           TOMO_F32, s)))
         return st;
     cudaEvent_t e[3];
     for (int k = 0; k < 3; ++k)
@@ -658,7 +659,7 @@ tomo_status tomo_autotune(tomo_ctx *ctx, const tomo_problem *prob,
     cudaStream_t s = (cudaStream_t)stream;
     if ((st = ensure_plane(ctx, &prob->cube, 1, kDefaultTiling)) ||
         (st = prepare_rays(ctx, &prob->cube, 1, &prob->img,
-                           prob->pointing_host, s)))
+                           prob->pointing_host, TOMO_F32, s)))
         return st;
     const int64_t nvox = (int64_t)prob->cube.nx * prob->cube.ny * prob->cube.nz;
     const int64_t npix = (int64_t)prob->img.n_img * prob->img.nu * prob->img.nv;
@@ -684,7 +685,8 @@ tomo_status tomo_autotune(tomo_ctx *ctx, const tomo_problem *prob,
             best.adj_ms = a;
         }
     }
-    best.rules = rules_for(ctx, &prob->cube, &prob->img);
+    best.rules = rules_for(ctx, &prob->cube, &prob->img,
+                           4 * (int64_t)prob->cube.nx);
     Tuned *entry = bucket_of(ctx, &prob->cube, &prob->img);
     if (entry)
         *entry = best;
@@ -751,7 +753,7 @@ tomo_status tomo_autotune(tomo_ctx *ctx, const tomo_problem *prob,
     entry->adj_ms = cur_a;
     // leave the cached hints on the winning rules
     if ((st = prepare_rays(ctx, &prob->cube, 1, &prob->img,
-                           prob->pointing_host, s)))
+                           prob->pointing_host, TOMO_F32, s)))
         return st;
     CUDA_TRY(ctx, cudaStreamSynchronize(s));
     if (best_out) {
@@ -781,7 +783,7 @@ tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
     tomo_status st;
     if (cube && ((st = check_cube(ctx, cube, 1)) || (st = check_img(ctx, img))))
         return st;
-    const tomo_plane_rules r = rules ? *rules : default_plane_rules(*cube);
+    const tomo_plane_rules r = rules ? *rules : default_plane_rules(*cube, kAnyRow);
     const double v[6] = { r.min_pitch, r.fwd_min_pitch, r.fwd_max_ratio,
                           r.general_ratio, r.fwd_group, r.adj_group };
     for (double x : v)

@@ -73,6 +73,10 @@ struct tomo_ctx {
     // the plane forward (a coarse host estimate): the per-ray forward then
     // runs in its listed form
     bool fwd_plane_all = false;
+    // whether every image of the geometry dense_key takes the plane forward
+    // from the lower default pitch on (stack_rules)
+    bool dense_valid = false, dense = false;
+    uint64_t dense_key = 0;
     // layouts (bit L) that some image of the cached geometry may walk in: in
     // P^T (or with every image plane by plane), and in the plane forward;
     // layout passes of the others are not launched, and with no layout at all
@@ -128,9 +132,12 @@ int reduce_grid(const tomo_ctx *ctx, int64_t n);
 // context's option.
 Tiling tiling_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
                   const tomo_image_geom *g);
-// Walk rules for a problem: its size bucket's, else the context's.
+// Walk rules for a problem: its size bucket's, else the context's, else the
+// defaults for the row that its forward gathers from (default_plane_rules);
+// *built_in: whether the defaults were taken.
 tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
-                           const tomo_image_geom *g);
+                           const tomo_image_geom *g, int64_t row = kAnyRow,
+                           bool *built_in = nullptr);
 void free_plan(tomo_ctx *ctx);
 // Single-problem P and P^T with the context's walk: plane-synchronous
 // (layout copies + plane kernels) when enabled and supported, else the
@@ -173,10 +180,12 @@ bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules);
-// Builds (or reuses) the context's ray records for one geometry on `s`.
+// Builds (or reuses) the context's ray records for one geometry on `s`; dtype:
+// of the cube that P reads (TOMO_F32 for calls without one).
 tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          int32_t n_frames, const tomo_image_geom *g,
-                         const tomo_pointing *ptg, cudaStream_t s);
+                         const tomo_pointing *ptg, tomo_dtype dtype,
+                         cudaStream_t s);
 
 #define CUDA_TRY(ctx, call)                                                  \
     do {                                                                     \

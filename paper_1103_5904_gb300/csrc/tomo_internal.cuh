@@ -69,28 +69,47 @@ constexpr double kPlaneMinPitch = 0.16;
 //    loop when lo < kPlaneFwdMaxRatio (0.81x the per-ray forward at lo = 0,
 //    0.94x at 0.017, 1.04x at 0.026), and whenever the pixels are at least
 //    kPlaneFwdMinPitch voxels apart, where the per-ray warps share few L1
-//    lines (1.22 against 2.14 ms at 1.07 voxel); from kPlaneLargeCube voxels
-//    on kPlaneFwdMinPitchLarge.  Per-ray over plane time of the every-slab
-//    body at 2 / 7 / 30 degrees of latitude: pixels 0.53 voxel apart, 64^3
-//    cube 0.91 / 0.92 / 1.21 (bf16 0.87 / 0.91 / 1.13), 128^3 1.08 / 1.18 /
-//    1.49 (0.99 / 1.09 / 1.38), 256^3 1.35 / 1.42 / 1.79 (1.21 / 1.28 / 1.60);
-//    0.35 apart, 128^3 0.96 / 1.05 / 1.34 (0.86 / 0.94 / 1.21); 0.8 apart,
-//    64^3 1.15 / 1.16 / 1.38.  128^3, 60 views of 256^2 within 7 degrees: 456
-//    -> 375 us.
+//    lines (1.22 against 2.14 ms at 1.07 voxel); on cubes of kPlaneLargeCube
+//    voxels and more from kPlaneFwdMinPitchLarge on, when a row of voxels is a
+//    whole number of kRowBytes.  The lanes of a per-ray warp read several rows
+//    of the cube at about the same x; with such rows they meet in the same L1
+//    banks, and the per-ray walk takes 1.2 to 1.5x its time on cubes a few
+//    voxels wider.  Per-ray over plane time (by address) at 2 and 7 degrees of
+//    latitude, pixels 0.5 / 0.6 / 0.74 voxel apart:
+//      float  128^3 1.10 1.16 / 1.25 1.31 / 1.30 1.36, 160^3 1.18 1.20 / 1.31
+//      1.36 / 1.42 1.58, 256^3 1.30 1.37 / 1.38 1.46 / 1.37 1.47; but 132^3
+//      0.94 1.00 / 0.93 0.99 / 0.90 0.96, 200^3 0.97 1.04 / 0.98 1.05 / 0.97
+//      1.03
+//      bf16   128^3 1.01 1.07 / 1.16 1.22 / 1.23 1.28, 256^3 1.13 1.21 / 1.26
+//      1.33 / 1.40 1.47; but 160^3 (320-byte rows) 0.88 0.90 / 0.90 0.95 /
+//      0.95 1.06, 200^3 0.88 0.95 / 0.89 0.95 / 0.89 0.94
+//    64^3: 0.91 / 0.92 (0.53 apart).  By offset (a cube across a multiple of
+//    2^32) the ratios are 10-14 % lower: 0.96 (bf16 0.91) at the very edge
+//    (128^3, 0.5 apart, 2 degrees), 1.0 to 1.4 above it.  Walks of two values
+//    per voxel and batched calls gain from 0.5 voxel on whatever the row: frame
+//    pairs 104^3 to 256^3 0.99-1.9, Thomson B 1.2-1.8, batches of 6 cubes of
+//    96^3 to 128^3 1.12-1.83.
 constexpr int32_t kPlaneFwdBit = 64;
 constexpr double kPlaneFwdMinPitch = 0.75;
 constexpr double kPlaneFwdMinPitchLarge = 0.5;
 constexpr int64_t kPlaneLargeCube = 1 << 20;
+constexpr int64_t kRowBytes = 128;
 constexpr double kPlaneFwdMaxRatio = 0.02;
 constexpr int32_t kPlaneGeneralBit = 128;
 constexpr double kPlaneGeneralRatio = 0.035;
+// Bytes of a row of voxels of the cube that a forward gathers from, for
+// default_plane_rules: kAnyRow for the walks that need no special row length,
+// kTimeRow for the time-interpolated walk on separate frames (two loads a frame
+// apart, by offset), which takes the plane forward from kPlaneFwdMinPitch only.
+constexpr int64_t kAnyRow = 0, kTimeRow = 1;
 // The thresholds above as walk rules of a cube (the default of every size
 // bucket that tomo_autotune or tomo_set_plane_rules has not set).
-inline tomo_plane_rules default_plane_rules(const tomo_cube_geom &c)
+inline tomo_plane_rules default_plane_rules(const tomo_cube_geom &c, int64_t row)
 {
     tomo_plane_rules r;
     r.min_pitch = kPlaneMinPitch;
-    r.fwd_min_pitch = (int64_t)c.nx * c.ny * c.nz >= kPlaneLargeCube
+    r.fwd_min_pitch = (int64_t)c.nx * c.ny * c.nz >= kPlaneLargeCube &&
+                              row % kRowBytes == 0
                           ? kPlaneFwdMinPitchLarge : kPlaneFwdMinPitch;
     r.fwd_max_ratio = kPlaneFwdMaxRatio;
     r.general_ratio = kPlaneGeneralRatio;

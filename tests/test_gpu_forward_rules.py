@@ -1,9 +1,12 @@
-"""Which forward a stack takes where no image takes the plane walk.
+"""Which forward the built-in walk rules choose.
 
 A pixel pitch just below the plane forward's threshold must cost what it
 cost without the plane walk: one per-ray launch, no layout copy and no launch
-that finds nothing to do (the walk is a matter of speed only: Section 3.3.1,
-Eq. lo)."""
+that finds nothing to do.  Tilted views with pixels 0.5 to 0.75 voxel apart
+take the plane forward only on large cubes and only where it takes every
+image; for one value per voxel, only where the rows of voxels are whole
+128-byte lines (elsewhere it measured up to 25 % slower).  The walk is a matter of speed only (Section
+3.3.1, Eq. lo)."""
 
 import numpy as np
 import pytest
@@ -54,4 +57,41 @@ def test_below_the_threshold_one_launch(T, kind, below):
     ctx.set_option(T.tomo.TOMO_OPT_PLANE_SYNC, 0)
     assert torch.equal(got, T.tomo_project(x, g, p, npx, npx, n_frames=frames,
                                            ctx=ctx))
+    ctx.close()
+
+
+@pytest.mark.parametrize("shape,dtype,frames,kind,plane", [
+    ((128, 128, 128), "f32", 1, "emission", True),
+    ((128, 128, 128), "bf16", 1, "emission", True),
+    ((101, 101, 101), "f32", 1, "emission", False),  # below 2^20 voxels
+    ((104, 104, 104), "f32", 1, "emission", False),  # 416-byte rows
+    ((127, 128, 128), "f32", 1, "emission", False),
+    ((160, 96, 96), "f32", 1, "emission", True),     # 640-byte rows
+    ((160, 96, 96), "bf16", 1, "emission", False),   # 320-byte rows
+    ((160, 96, 96), "bf16", 1, "pB", True),          # walks floats
+    ((104, 104, 104), "f32", 2, "emission", True),   # frame pairs
+    ((104, 104, 104), "f32", 1, "B", True),          # one walk, two values
+])
+def test_default_forward(T, shape, dtype, frames, kind, plane):
+    nx, ny, nz = shape
+    npx = 16
+    g, p = synth.cube_geom(nx, 1.5, ny, nz), _views(nx, npx, 0.6, n_img=2)
+    p[:, 1] = np.deg2rad([97.0, 263.0])  # along y: image rows along x
+    x = torch.ones(((frames,) if frames > 1 else ()) + (nz, ny, nx),
+                   device="cuda")
+    x = x.to(torch.bfloat16) if dtype == "bf16" else x
+    ctx = T.Context()
+    for pitch, want in ((0.6, plane), (0.45, False), (0.8, True)):
+        p[:, 4:6] = np.arctan(pitch * (3.0 / nx) / 215.0)
+        T.tomo_project(x, g, p, npx, npx, n_frames=frames, kind=kind, ctx=ctx)
+        code = T.tomo_walk_plan(len(p), ctx=ctx)
+        assert (((code & 2) != 0) == want).all(), (pitch, code)
+    # one image below 0.5 voxel: each is held to 0.75 voxel, but where one
+    # launch walks both kinds of image
+    p[0, 4:6] = np.arctan(0.45 * (3.0 / nx) / 215.0)
+    for pitch, want in ((0.6, kind == "B"), (0.8, True)):
+        p[1, 4:6] = np.arctan(pitch * (3.0 / nx) / 215.0)
+        T.tomo_project(x, g, p, npx, npx, n_frames=frames, kind=kind, ctx=ctx)
+        code = T.tomo_walk_plan(len(p), ctx=ctx)
+        assert ((code & 2) != 0).tolist() == [False, want], (pitch, code)
     ctx.close()
