@@ -219,10 +219,6 @@ static bool use_one_b(const tomo_ctx *ctx, const tomo_image_geom *g,
     return g->kind == TOMO_KIND_B && n_frames == 1 && (ctx->channels & 2);
 }
 
-// Far above the rounding of the host's and the device's sines and products
-// (1e-15), far below any difference that matters for speed.
-constexpr double kHintTol = 1e-9;
-
 // The row that P gathers from, as default_plane_rules takes it.
 static int64_t forward_row(const tomo_ctx *ctx, const tomo_cube_geom *c,
                            int32_t n_frames, const tomo_image_geom *g,
@@ -284,10 +280,7 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                     use_one_b(ctx, g, n_frames), h);
     const uint64_t hh = fnv1a(h, &rules, sizeof(rules));
     tomo_status st;
-    if ((st = ensure(ctx, ctx->layout_used, sizeof(unsigned))) ||
-        (st = ensure(ctx, ctx->per_ray_fwd,
-                     sizeof(unsigned) * (1 + (size_t)g->n_img))))
-        return st;
+    if ((st = ensure(ctx, ctx->layout_used, sizeof(unsigned)))) return st;
     if (ctx->ray_cache && ctx->key_valid && ctx->key == h) {
         if (ctx->hint_key == hh) {
             CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->setup_done, 0));
@@ -298,7 +291,6 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
         ctx->key_valid = false;
         CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->setup_done, 0));
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->layout_used.p, 0, sizeof(unsigned), s));
-        CUDA_TRY(ctx, cudaMemsetAsync(ctx->per_ray_fwd.p, 0, sizeof(unsigned), s));
         estimate_walks(ctx, c, g, ptg, rules);
         LAUNCH(ctx, TOMO_K_SETUP, s,
                launch_frames((const tomo_pointing *)ctx->ptg.p, g->n_img, g->nu,
@@ -306,8 +298,7 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                              (double *)ctx->tan_u.p, (double *)ctx->tan_v.p,
                              (ImgParam *)ctx->params.p,
                              make_double3(c->dx, c->dy, c->dz),
-                             (unsigned *)ctx->layout_used.p,
-                             (unsigned *)ctx->per_ray_fwd.p, rules, s));
+                             (unsigned *)ctx->layout_used.p, rules, s));
         CUDA_TRY(ctx, cudaEventRecord(ctx->setup_done, s));
         ctx->hint_key = hh;
         ctx->key_valid = true;
@@ -326,7 +317,6 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
     CUDA_TRY(ctx, cudaMemcpyAsync(ctx->ptg.p, ptg, sizeof(tomo_pointing) * n_img,
                                   cudaMemcpyHostToDevice, s));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->layout_used.p, 0, sizeof(unsigned), s));
-    CUDA_TRY(ctx, cudaMemsetAsync(ctx->per_ray_fwd.p, 0, sizeof(unsigned), s));
     estimate_walks(ctx, c, g, ptg, rules);
     LAUNCH(ctx, TOMO_K_SETUP, s,
            launch_frames((const tomo_pointing *)ctx->ptg.p, g->n_img, g->nu,
@@ -334,8 +324,7 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          (double *)ctx->tan_u.p, (double *)ctx->tan_v.p,
                          (ImgParam *)ctx->params.p,
                          make_double3(c->dx, c->dy, c->dz),
-                         (unsigned *)ctx->layout_used.p,
-                         (unsigned *)ctx->per_ray_fwd.p, rules, s));
+                         (unsigned *)ctx->layout_used.p, rules, s));
     LAUNCH(ctx, TOMO_K_SETUP, s,
            launch_ray_setup((const Frame *)ctx->frames.p,
                             (const double *)ctx->tan_u.p,
@@ -394,37 +383,13 @@ tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
     return default_plane_rules(*c, row);
 }
 
-// The device's rules (hint.cuh) evaluated from the boresight, with margins
-// towards "may"; the pixel pitch with the smallest voxel side.
-bool plane_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
-                    const tomo_plane_rules &r)
-{
-    const double dmin = fmin(c->dx, fmin(c->dy, c->dz));
-    return p.d_obs * fabs(tan(p.cdelt_u)) / dmin >= 0.9 * r.min_pitch;
-}
-
-bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
-                            const tomo_plane_rules &r)
-{
-    if (!plane_estimate(p, c, r)) return false;
-    const double cl = cos(p.lat);
-    const double w[3] = { fabs(cl * cos(p.lon)), fabs(cl * sin(p.lon)),
-                          fabs(sin(p.lat)) };
-    const double hi = fmax(w[0], fmax(w[1], w[2]));
-    const double lo = fmin(w[0], fmin(w[1], w[2])) / hi;
-    const double dmin = fmin(c->dx, fmin(c->dy, c->dz));
-    const double pitch = p.d_obs * fabs(tan(p.cdelt_u)) / dmin;
-    return pitch >= 0.9 * r.fwd_min_pitch || lo < 1.5 * r.fwd_max_ratio;
-}
-
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules)
 {
-    ctx->fwd_plane_all = ctx->fwd_plane_sure = true;
+    ctx->fwd_plane_sure = true;
     ctx->lay_adj = ctx->lay_fwd = 0u;
     for (int32_t i = 0; i < g->n_img; ++i) {
-        ctx->fwd_plane_all &= plane_forward_estimate(ptg[i], c, rules);
         const PlaneHint h = plane_hint(ptg[i], image_frame(ptg[i]), g->nu, g->nv,
                                        make_double3(c->dx, c->dy, c->dz), rules,
                                        kHintTol);
@@ -500,14 +465,6 @@ int plane_group(const tomo_ctx *ctx, const tomo_cube_geom *c,
     return n_acc > 1 ? n_img : 8;
 }
 
-// The per-ray forward's image list when the host estimate says every image
-// may take the plane forward (the list is then short or empty), else NULL:
-// images certain to need the per-ray walk keep its one-CTA-per-tile grid.
-const unsigned *per_ray_list(const tomo_ctx *ctx)
-{
-    return ctx->fwd_plane_all ? (const unsigned *)ctx->per_ray_fwd.p : nullptr;
-}
-
 tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
                         int32_t n_frames, const uint8_t *mask, float *out,
                         const tomo_cube_geom *c, const tomo_image_geom *g,
@@ -538,8 +495,7 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
             LAUNCH(ctx, TOMO_K_FORWARD, s,
                    launch_forward(rays, prm, cube_dev, dtype, fstride, true,
                                   mask, out, g->n_img, g->nu, g->nv, c->nx,
-                                  c->nx * c->ny, t, done, s, true,
-                                  per_ray_list(ctx), ctx->num_sms));
+                                  c->nx * c->ny, t, done, s, true));
         LAUNCH(ctx, TOMO_K_FORWARD, s,
                launch_forward_plane_pair(
                    rays, prm, pc, n_frames - 1, cube_dev, dtype, fstride, mask, out,
@@ -563,7 +519,7 @@ tomo_status forward_one(tomo_ctx *ctx, const void *cube_dev, tomo_dtype dtype,
                    launch_forward(rays, prm, cube_dev, dtype, fstride,
                                   n_frames > 1, mask, out, g->n_img, g->nu,
                                   g->nv, c->nx, c->nx * c->ny, t, done, s,
-                                  true, per_ray_list(ctx), ctx->num_sms));
+                                  true));
         LAUNCH(ctx, TOMO_K_FORWARD, s,
                launch_forward_plane(
                    rays, prm, pc, dtype, fstride, n_frames > 1, mask, out,
@@ -905,7 +861,6 @@ void tomo_destroy(tomo_ctx *ctx)
                        &ctx->params, &ctx->rays, &ctx->b, &ctx->r, &ctx->p,
                        &ctx->q, &ctx->t, &ctx->p16, &ctx->S, &ctx->partials,
                        &ctx->counter, &ctx->count64, &ctx->layout_used,
-                       &ctx->per_ray_fwd,
                        &ctx->lay1, &ctx->lay2, &ctx->mcube, &ctx->rho2,
                        &ctx->thf, &ctx->th1, &ctx->th2, &ctx->thimg,
                        &ctx->pr[0], &ctx->pr[1], &ctx->pr[2] };

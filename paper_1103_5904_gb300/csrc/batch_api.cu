@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "batch.cuh"
+#include "hint.cuh"
 #include "host.h"
 
 using namespace tomo;
@@ -196,16 +197,18 @@ tomo_status prepare_batch(tomo_ctx *ctx, int32_t n, const tomo_problem *probs,
                               ((g.nv + P->tl[i].tile_v - 1) / P->tl[i].tile_v);
         P->tile_prefix[i + 1] = P->tile_prefix[i] + tiles;
         bool plane_ok = false;
-        const tomo_plane_rules rules = rules_for(ctx, &probs[i].cube, &g);
-        for (int32_t k = 0; k < g.n_img; ++k)
-            plane_ok |= plane_estimate(probs[i].pointing_host[k],
-                                       &probs[i].cube, rules);
+        const tomo_cube_geom &c = probs[i].cube;
+        const tomo_plane_rules rules = rules_for(ctx, &c, &g);
+        for (int32_t k = 0; k < g.n_img && !plane_ok; ++k)
+            plane_ok = plane_hint(probs[i].pointing_host[k],
+                                  image_frame(probs[i].pointing_host[k]), g.nu,
+                                  g.nv, make_double3(c.dx, c.dy, c.dz), rules,
+                                  kHintTol).layouts != 0u;
         P->ptile_prefix[i + 1] =
             P->ptile_prefix[i] + (plane_ok ? (int64_t)g.n_img *
                                      ((g.nu + kPlaneTileU - 1) / kPlaneTileU) *
                                      ((g.nv + kPlaneTileV - 1) / kPlaneTileV) : 0);
         P->rtile_prefix[i + 1] = P->rtile_prefix[i] + (plane_ok ? 0 : tiles);
-        const tomo_cube_geom &c = probs[i].cube;
         P->vox_off[i + 1] = P->vox_off[i] + (int64_t)c.nx * c.ny * c.nz;
         for (int L = 1; L <= 2; ++L) {
             const int64_t nb = L == 1 ? c.ny : c.nz, nc = L == 1 ? c.nz : c.ny;
@@ -249,7 +252,7 @@ tomo_status prepare_batch(tomo_ctx *ctx, int32_t n, const tomo_problem *probs,
                launch_frames((const tomo_pointing *)P->ptg.p + P->img_off[i],
                              p.img.n_img, p.img.nu, p.img.nv, 1, fr, tu, tv, pr,
                              make_double3(p.cube.dx, p.cube.dy, p.cube.dz),
-                             (unsigned *)P->lay_used.p + i, nullptr,
+                             (unsigned *)P->lay_used.p + i,
                              rules_for(ctx, &p.cube, &p.img), s));
         LAUNCH(ctx, TOMO_K_SETUP, s,
                launch_ray_setup(fr, tu, tv, cube_dev(&p.cube), p.img.n_img,

@@ -66,13 +66,6 @@ struct tomo_ctx {
     tomo::host::DevBuf ptg, frames, tan_u, tan_v, params, rays;
     // bit L set: some image of the cached geometry walks in layout L
     tomo::host::DevBuf layout_used;
-    // { count, image indices }: the images of the cached geometry whose hint
-    // leaves them to the per-ray forward
-    tomo::host::DevBuf per_ray_fwd;
-    // every image of the cached geometry lies above or near the threshold of
-    // the plane forward (a coarse host estimate): the per-ray forward then
-    // runs in its listed form
-    bool fwd_plane_all = false;
     // whether every image of the geometry dense_key takes the plane forward
     // from the lower default pitch on (stack_rules)
     bool dense_valid = false, dense = false;
@@ -132,6 +125,10 @@ int reduce_grid(const tomo_ctx *ctx, int64_t n);
 // context's option.
 Tiling tiling_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
                   const tomo_image_geom *g);
+// Tolerance of plane_hint on the host: far above the rounding of the host's
+// and the device's sines and products (1e-15), far below any difference that
+// matters for speed.
+constexpr double kHintTol = 1e-9;
 // Walk rules for a problem: its size bucket's, else the context's, else the
 // defaults for the row that its forward gathers from (default_plane_rules);
 // *built_in: whether the defaults were taken.
@@ -166,17 +163,9 @@ tomo_status adjoint_one(tomo_ctx *ctx, const float *images,
                         const tomo_cube_geom *c, int32_t n_frames,
                         const tomo_image_geom *g, Tiling t,
                         const double *done, cudaStream_t s);
-// Coarse host estimates, from the boresight and with wide margins, of whether
-// an image may get a valid hint and whether it lies above or near the
-// thresholds of the plane forward.  Only speed depends on them: they choose
-// between kernels that read the device's hints themselves.
-bool plane_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
-                    const tomo_plane_rules &r);
-bool plane_forward_estimate(const tomo_pointing &p, const tomo_cube_geom *c,
-                            const tomo_plane_rules &r);
-// Fills the context's per-geometry schedule: from plane_hint with a tolerance,
-// the layouts whose passes are launched and whether the per-ray forward is
-// (results depend on these); from the estimate above, its listed form.
+// Fills the context's per-geometry schedule from plane_hint with a tolerance:
+// the layouts whose passes are launched and whether the per-ray forward is.
+// Results depend on these.
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules);
