@@ -452,6 +452,15 @@ tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
                                  const tomo_image_geom *img,
                                  const tomo_plane_rules *rules);
 
+/* The same for some of the rules: those whose bit is set in `fields` (bit k:
+ * the k-th member of tomo_plane_rules); the others keep the built-in defaults,
+ * which depend on the cube and the walk.  tomo_set_plane_rules sets all six. */
+tomo_status tomo_set_plane_rule_fields(tomo_ctx *ctx,
+                                       const tomo_cube_geom *cube,
+                                       const tomo_image_geom *img,
+                                       const tomo_plane_rules *rules,
+                                       uint32_t fields);
+
 /* The walk chosen for each image of the most recent single-problem
  * geometry by the single-value P and P^T (a report of the schedule, no
  * counterpart in the paper; synchronises the legacy default stream).  It

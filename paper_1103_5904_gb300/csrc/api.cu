@@ -245,9 +245,12 @@ static tomo_plane_rules stack_rules(tomo_ctx *ctx, const tomo_cube_geom *c,
                                     const tomo_pointing *ptg, int64_t row,
                                     bool one_walk, uint64_t geom)
 {
-    bool built_in;
-    tomo_plane_rules r = rules_for(ctx, c, g, row, &built_in);
-    if (!built_in || one_walk || r.fwd_min_pitch != kPlaneFwdMinPitchLarge) return r;
+    uint32_t set;
+    tomo_plane_rules r = rules_for(ctx, c, g, row, &set);
+    if ((set & kRuleFwdMinPitch) || one_walk ||
+        r.fwd_min_pitch != kPlaneFwdMinPitchLarge)
+        return r;
+    geom = fnv1a(geom, &r, sizeof(r));
     if (!ctx->dense_valid || ctx->dense_key != geom) {
         ctx->dense = true;
         for (int32_t i = 0; i < g->n_img && ctx->dense; ++i)
@@ -371,16 +374,27 @@ Tiling tiling_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
 }
 
 tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
-                           const tomo_image_geom *g, int64_t row, bool *built_in)
+                           const tomo_image_geom *g, int64_t row, uint32_t *fields)
 {
-    if (built_in) *built_in = false;
+    const tomo_plane_rules *from = &ctx->rules;
+    uint32_t set = ctx->rule_fields;
     for (const Tuned &t : ctx->tuned)
         if (t.nx == c->nx && t.ny == c->ny && t.nz == c->nz && t.nu == g->nu &&
-            t.nv == g->nv)
-            return t.rules;
-    if (ctx->rules_set) return ctx->rules;
-    if (built_in) *built_in = true;
-    return default_plane_rules(*c, row);
+            t.nv == g->nv) {
+            from = &t.rules;
+            set = t.fields;
+            break;
+        }
+    if (fields) *fields = set;
+    if (set == kAllRules) return *from;
+    tomo_plane_rules r = default_plane_rules(*c, row);
+    if (set & 1u) r.min_pitch = from->min_pitch;
+    if (set & kRuleFwdMinPitch) r.fwd_min_pitch = from->fwd_min_pitch;
+    if (set & 4u) r.fwd_max_ratio = from->fwd_max_ratio;
+    if (set & 8u) r.general_ratio = from->general_ratio;
+    if (set & 16u) r.fwd_group = from->fwd_group;
+    if (set & 32u) r.adj_group = from->adj_group;
+    return r;
 }
 
 void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,

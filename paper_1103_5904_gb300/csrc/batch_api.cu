@@ -690,6 +690,7 @@ tomo_status tomo_autotune(tomo_ctx *ctx, const tomo_problem *prob,
     }
     best.rules = rules_for(ctx, &prob->cube, &prob->img,
                            4 * (int64_t)prob->cube.nx);
+    best.fields = kAllRules;
     Tuned *entry = bucket_of(ctx, &prob->cube, &prob->img);
     if (entry)
         *entry = best;
@@ -770,31 +771,31 @@ tomo_status tomo_autotune(tomo_ctx *ctx, const tomo_problem *prob,
     return TOMO_OK;
 }
 
-tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
-                                 const tomo_image_geom *img,
-                                 const tomo_plane_rules *rules)
+tomo_status tomo_set_plane_rule_fields(tomo_ctx *ctx, const tomo_cube_geom *cube,
+                                       const tomo_image_geom *img,
+                                       const tomo_plane_rules *rules,
+                                       uint32_t fields)
 {
     if (!ctx) return TOMO_ERR_ARG;
     ctx->err[0] = 0;
     if ((cube == nullptr) != (img == nullptr))
         return fail(ctx, TOMO_ERR_ARG, "cube and img must both be given or "
                                        "both be NULL");
-    if (!cube && !rules) {
-        ctx->rules_set = false;
-        return TOMO_OK;
-    }
+    if (fields & ~kAllRules)
+        return fail(ctx, TOMO_ERR_ARG, "unknown rule fields 0x%x", fields);
+    if (!rules) fields = 0;
     tomo_status st;
     if (cube && ((st = check_cube(ctx, cube, 1)) || (st = check_img(ctx, img))))
         return st;
-    const tomo_plane_rules r = rules ? *rules : default_plane_rules(*cube, kAnyRow);
+    const tomo_plane_rules r = rules ? *rules : tomo_plane_rules{};
     const double v[6] = { r.min_pitch, r.fwd_min_pitch, r.fwd_max_ratio,
                           r.general_ratio, r.fwd_group, r.adj_group };
-    for (double x : v)
-        if (!(x >= 0.0) || isnan(x))
+    for (int k = 0; k < 6; ++k)
+        if (((fields >> k) & 1u) && (!(v[k] >= 0.0) || isnan(v[k])))
             return fail(ctx, TOMO_ERR_ARG, "plane rules must be >= 0");
     if (!cube) {
         ctx->rules = r;
-        ctx->rules_set = true;
+        ctx->rule_fields = fields;
         return TOMO_OK;
     }
     Tuned *e = bucket_of(ctx, cube, img);
@@ -811,7 +812,15 @@ tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
         e = &ctx->tuned.back();
     }
     e->rules = r;
+    e->fields = fields;
     return TOMO_OK;
+}
+
+tomo_status tomo_set_plane_rules(tomo_ctx *ctx, const tomo_cube_geom *cube,
+                                 const tomo_image_geom *img,
+                                 const tomo_plane_rules *rules)
+{
+    return tomo_set_plane_rule_fields(ctx, cube, img, rules, kAllRules);
 }
 
 tomo_status tomo_project_batched(tomo_ctx *ctx, int32_t n,

@@ -27,7 +27,12 @@ struct Tuned {
     Tiling tl;
     float fwd_ms, adj_ms;
     tomo_plane_rules rules;
+    // rules that are set (bit k: the k-th member of tomo_plane_rules); the
+    // others are the built-in defaults
+    uint32_t fields;
 };
+// Bits of Tuned::fields.
+constexpr uint32_t kRuleFwdMinPitch = 2u, kAllRules = 63u;
 
 struct BatchPlan;  // batch_api.cu
 
@@ -51,10 +56,10 @@ struct tomo_ctx {
     // side; bit 1: Thomson B in one walk on (m' x, m x) pairs
     int channels = 3;
     tomo::Tiling tiling = { 32, 8, 8 };
-    // walk rules of size buckets without their own, once set by the caller
-    // (else the built-in defaults of the bucket's cube)
+    // walk rules of size buckets without their own, as far as set by the
+    // caller (as in Tuned)
     tomo_plane_rules rules = {};
-    bool rules_set = false;
+    uint32_t rule_fields = 0;
     // geometry cache
     bool key_valid = false;
     uint64_t key = 0;       // geometry of the cached ray records
@@ -129,12 +134,12 @@ Tiling tiling_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
 // and the device's sines and products (1e-15), far below any difference that
 // matters for speed.
 constexpr double kHintTol = 1e-9;
-// Walk rules for a problem: its size bucket's, else the context's, else the
-// defaults for the row that its forward gathers from (default_plane_rules);
-// *built_in: whether the defaults were taken.
+// Walk rules for a problem: the set ones of its size bucket's, if it has an
+// entry, else of the context's; for the others the defaults for the row that
+// its forward gathers from (default_plane_rules).  *fields: those that are set.
 tomo_plane_rules rules_for(const tomo_ctx *ctx, const tomo_cube_geom *c,
                            const tomo_image_geom *g, int64_t row = kAnyRow,
-                           bool *built_in = nullptr);
+                           uint32_t *fields = nullptr);
 void free_plan(tomo_ctx *ctx);
 // Single-problem P and P^T with the context's walk: plane-synchronous
 // (layout copies + plane kernels) when enabled and supported, else the

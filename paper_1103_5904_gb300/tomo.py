@@ -146,6 +146,10 @@ _SIGNATURES = {
     "tomo_set_plane_rules": (C.c_int, [_VP, C.POINTER(CubeGeom),
                                        C.POINTER(ImageGeom),
                                        C.POINTER(PlaneRules)]),
+    "tomo_set_plane_rule_fields": (C.c_int, [_VP, C.POINTER(CubeGeom),
+                                             C.POINTER(ImageGeom),
+                                             C.POINTER(PlaneRules),
+                                             C.c_uint32]),
     "tomo_walk_plan": (C.c_int, [_VP, C.c_int32, C.POINTER(C.c_int32)]),
     "tomo_project_batched": (C.c_int, [_VP, C.c_int32, C.POINTER(Problem),
                                        _VP]),
@@ -606,24 +610,19 @@ def tomo_set_plane_rules(rules=None, geom=None, nu=None, nv=None,
     ``geom`` and ``nu`` x ``nv`` images, or the context's default when
     ``geom`` is None."""
     ctx = _ctx(ctx)
-    r = None
+    r, fields = None, 0
     if rules is not None:
-        d = {"min_pitch": 0.16, "fwd_min_pitch": 0.75, "fwd_max_ratio": 0.02,
-             "general_ratio": 0.035, "fwd_group": 0.0, "adj_group": 0.0}
-        if geom is not None and \
-                int(geom["nx"]) * int(geom["ny"]) * int(geom["nz"]) >= 1 << 20:
-            d["fwd_min_pitch"] = 0.5
         unknown = set(rules) - set(RULE_FIELDS)
         if unknown:
             raise ValueError("unknown rule(s) %s" % sorted(unknown))
-        d.update(rules)
-        r = PlaneRules(*[float(d[f]) for f in RULE_FIELDS])
+        r = PlaneRules(*[float(rules.get(f, 0.0)) for f in RULE_FIELDS])
+        fields = sum(1 << k for k, f in enumerate(RULE_FIELDS) if f in rules)
     cg = ig = None
     if geom is not None:
         cg = C.byref(cube_geom_struct(geom))
         ig = C.byref(ImageGeom(int(n_img), int(nu), int(nv)))
-    ctx.check(load_library().tomo_set_plane_rules(
-        ctx.handle, cg, ig, None if r is None else C.byref(r)))
+    ctx.check(load_library().tomo_set_plane_rule_fields(
+        ctx.handle, cg, ig, None if r is None else C.byref(r), fields))
 
 
 def tomo_walk_plan(n_img, ctx=None):

@@ -95,3 +95,34 @@ def test_default_forward(T, shape, dtype, frames, kind, plane):
         code = T.tomo_walk_plan(len(p), ctx=ctx)
         assert ((code & 2) != 0).tolist() == [False, want], (pitch, code)
     ctx.close()
+
+
+@pytest.mark.parametrize("bucket", [False, True], ids=["context", "bucket"])
+def test_other_rules_keep_the_default_forward(T, bucket):
+    """Setting one rule leaves the others at the built-in defaults of each
+    cube, for the context as for a size bucket; setting all of them does not."""
+    npx, ctx = 16, T.Context()
+    for n, plane in ((128, True), (104, False)):
+        g, p = synth.cube_geom(n, 1.5), _views(n, npx, 0.6, n_img=2)
+        x = torch.ones((n,) * 3, device="cuda")
+
+        def forward(rules):
+            at = (g, npx, npx, 2) if bucket else ()
+            T.tomo_set_plane_rules(rules, *at, ctx=ctx)
+            T.tomo_project(x, g, p, npx, npx, ctx=ctx)
+            code = T.tomo_walk_plan(len(p), ctx=ctx)
+            assert ((code & 2) != 0).all() or not ((code & 2) != 0).any()
+            return bool(code[0] & 2), bool(code[0] & 4)
+
+        assert forward(None) == (plane, True)
+        assert forward({"general_ratio": 1e30}) == (plane, False)
+        assert forward({"fwd_group": 8.0}) == (plane, True)
+        assert forward({"fwd_min_pitch": 0.55}) == (True, True)
+        every = {"min_pitch": 0.16, "fwd_min_pitch": 0.75, "fwd_max_ratio": 0.02,
+                 "general_ratio": 0.035, "fwd_group": 0.0, "adj_group": 0.0}
+        assert forward(every) == (False, True)
+        assert forward(None) == (plane, True)
+    for bad in ({"min_pitch": -1.0}, {"general_ratio": float("nan")}):
+        with pytest.raises(T.TomoError):
+            T.tomo_set_plane_rules(bad, ctx=ctx)
+    ctx.close()
