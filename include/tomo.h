@@ -162,7 +162,10 @@ typedef struct tomo_ctx tomo_ctx;
                                   addresses voxels by 32-bit byte offsets),
                                   else the per-ray walk is used.  Costs two
                                   cube-sized float buffers (times the
-                                  frames) of workspace. */
+                                  frames) of workspace; a new buffer of at
+                                  most 2^31 bytes may be held twice for a
+                                  moment, to place it between two multiples
+                                  of 2^32 (also for TOMO_OPT_CHANNELS). */
 #define TOMO_OPT_CHANNELS   8  /* bit mask (default 3) of the two-value
                                   plane walks: bit 0, time-interpolated P
                                   and P^T walk frame pairs (X[k], X[k+1])

@@ -55,12 +55,19 @@ tomo_status ensure(tomo_ctx *ctx, DevBuf &b, size_t bytes)
 
 // ensure() for a buffer that the gathering walks address by units of `unit`
 // bytes: a new allocation with a unit across a multiple of 2^32 (near_buffers)
-// is tried once more elsewhere.  Only speed depends on the outcome.
+// is tried once more elsewhere.  Only speed depends on the outcome.  Both
+// buffers are held for a moment, so only one of at most 2^31 bytes is tried
+// again: it then lies well at least every other time, where one of nearly 2^32
+// bytes or of many units hardly ever does.
+constexpr size_t kNearRetryBytes = (size_t)1 << 31;
+
 static tomo_status ensure_near(tomo_ctx *ctx, DevBuf &b, size_t bytes, size_t unit)
 {
     if (b.bytes >= bytes && b.p) return TOMO_OK;
     tomo_status st = ensure(ctx, b, bytes);
-    if (st || unit == 0 || near_buffers(b.p, unit, (int)(bytes / unit))) return st;
+    if (st || unit == 0 || bytes > kNearRetryBytes ||
+        near_buffers(b.p, unit, (int)(bytes / unit)))
+        return st;
     void *p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -429,7 +436,8 @@ tomo_status ensure_plane(tomo_ctx *ctx, const tomo_cube_geom *c,
     const size_t bytes =
         sizeof(float) * (size_t)c->nx * c->ny * c->nz * (size_t)n_frames;
     tomo_status st;
-    const size_t unit = bytes / (size_t)n_frames;
+    // (time-interpolated walks on separate frames go by offset)
+    const size_t unit = n_frames == 1 ? bytes : 0;
     if ((st = ensure_near(ctx, ctx->lay1, bytes, unit)) ||
         (st = ensure_near(ctx, ctx->lay2, bytes, unit)))
         return st;
