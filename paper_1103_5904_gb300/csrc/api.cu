@@ -276,7 +276,7 @@ static tomo_plane_rules stack_rules(tomo_ctx *ctx, const tomo_cube_geom *c,
 tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          int32_t n_frames, const tomo_image_geom *g,
                          const tomo_pointing *ptg, tomo_dtype dtype,
-                         cudaStream_t s)
+                         cudaStream_t s, bool without_p)
 {
     uint64_t h = 1469598103934665603ull;
     const int32_t cn[4] = { c->nx, c->ny, c->nz, n_frames };
@@ -285,10 +285,20 @@ tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
     h = fnv1a(h, cv, sizeof(cv));
     h = fnv1a(h, g, sizeof(*g));
     h = fnv1a(h, ptg, sizeof(tomo_pointing) * (size_t)g->n_img);
-    const tomo_plane_rules rules =
-        stack_rules(ctx, c, g, ptg, forward_row(ctx, c, n_frames, g, dtype),
-                    use_one_b(ctx, g, n_frames), h);
-    const uint64_t hh = fnv1a(h, &rules, sizeof(rules));
+    auto rules_of = [&](tomo_dtype type) {
+        return stack_rules(ctx, c, g, ptg, forward_row(ctx, c, n_frames, g, type),
+                           use_one_b(ctx, g, n_frames), h);
+    };
+    tomo_plane_rules rules = rules_of(dtype);
+    uint64_t hh = fnv1a(h, &rules, sizeof(rules));
+    if (without_p && ctx->hint_key != hh) {
+        const tomo_plane_rules other = rules_of(TOMO_BF16);
+        const uint64_t ho = fnv1a(h, &other, sizeof(other));
+        if (ctx->hint_key == ho) {
+            rules = other;
+            hh = ho;
+        }
+    }
     tomo_status st;
     if ((st = ensure(ctx, ctx->layout_used, sizeof(unsigned)))) return st;
     if (ctx->ray_cache && ctx->key_valid && ctx->key == h) {
@@ -1090,7 +1100,8 @@ tomo_status tomo_backproject(tomo_ctx *ctx, const tomo_cube_geom *cube,
     if (img->n_img == 0) return TOMO_OK;
     const Tiling tl = tiling_for(ctx, cube, img);
     if ((st = ensure_plane(ctx, cube, n_frames, tl)) ||
-        (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, TOMO_F32, s)))
+        (st = prepare_rays(ctx, cube, n_frames, img, pointing_host, TOMO_F32, s,
+                            true)))
         return st;
     if (img->kind != TOMO_KIND_EMISSION) {
         // dst += K T^T y: the Thomson epilogue skips the excluded voxels
@@ -1164,7 +1175,7 @@ tomo_status tomo_count_segments(tomo_ctx *ctx, const tomo_cube_geom *cube,
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return fail(ctx, TOMO_ERR_CUDA, "cannot select device");
     cudaStream_t s = (cudaStream_t)stream;
-    if ((st = prepare_rays(ctx, cube, 1, img, pointing_host, TOMO_F32, s))) return st;
+    if ((st = prepare_rays(ctx, cube, 1, img, pointing_host, TOMO_F32, s, true))) return st;
     if ((st = ensure(ctx, ctx->count64, sizeof(unsigned long long)))) return st;
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->count64.p, 0, sizeof(unsigned long long), s));
     LAUNCH(ctx, TOMO_K_FORWARD, s, launch_count((const RayRec *)ctx->rays.p, mask_dev, img->n_img,

@@ -175,11 +175,12 @@ void estimate_walks(tomo_ctx *ctx, const tomo_cube_geom *c,
                     const tomo_image_geom *g, const tomo_pointing *ptg,
                     const tomo_plane_rules &rules);
 // Builds (or reuses) the context's ray records for one geometry on `s`; dtype:
-// of the cube that P reads (TOMO_F32 for calls without one).
+// of the cube that P reads.  without_p: the call has no P and takes hints that
+// were built for another type as they are.
 tomo_status prepare_rays(tomo_ctx *ctx, const tomo_cube_geom *c,
                          int32_t n_frames, const tomo_image_geom *g,
                          const tomo_pointing *ptg, tomo_dtype dtype,
-                         cudaStream_t s);
+                         cudaStream_t s, bool without_p = false);
 
 #define CUDA_TRY(ctx, call)                                                  \
     do {                                                                     \

@@ -126,3 +126,22 @@ def test_other_rules_keep_the_default_forward(T, bucket):
         with pytest.raises(T.TomoError):
             T.tomo_set_plane_rules(bad, ctx=ctx)
     ctx.close()
+
+
+def test_transpose_keeps_the_hints_of_the_forward(T):
+    """A transpose between two forwards of a bf16 cube whose type decides the
+    forward (320-byte rows) rebuilds nothing."""
+    npx, ctx = 16, T.Context()
+    g, p = synth.cube_geom(160, 1.5, 96, 96), _views(160, npx, 0.6, n_img=2)
+    p[:, 1] = np.deg2rad([97.0, 263.0])  # along y: image rows along x
+    x = torch.ones((96, 96, 160), device="cuda", dtype=torch.bfloat16)
+    y = T.tomo_project(x, g, p, npx, npx, ctx=ctx)
+    code = T.tomo_walk_plan(len(p), ctx=ctx)
+    ctx.profile(reset=True)
+    T.tomo_backproject(y, g, p, ctx=ctx)
+    T.tomo_project(x, g, p, npx, npx, ctx=ctx)
+    assert ctx.profile(reset=True)["setup"][0] == 0
+    assert (T.tomo_walk_plan(len(p), ctx=ctx) == code).all()
+    T.tomo_project(x.float(), g, p, npx, npx, ctx=ctx)
+    assert ctx.profile(reset=True)["setup"][0] == 1  # the hints alone
+    ctx.close()
