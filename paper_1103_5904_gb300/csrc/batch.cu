@@ -376,9 +376,11 @@ __device__ __forceinline__ void vec_group(int64_t c0, int64_t c1, int g, const F
 // FP64 additions of block_sums: 8 problems (31^3 to 96^3), 10 iterations, took
 // 4.08 ms with chunks of 16384 elements, one kernel for all passes (64-bit
 // divisions and a run-time choice of pass per element) and separate kernels
-// for the scalar steps, and take 2.81 ms.
+// for the scalar steps, and take 2.81 ms.  At six CTAs per SM (40 registers) a
+// prior pass spills 28 bytes and the first residual 8; the update, 72 there, 40
+// at five (19.3 -> 17.8 us a pass).
 template <int kOp>
-__global__ void __launch_bounds__(kThreads, 6)
+__global__ void __launch_bounds__(kThreads, kOp == V_UPDATE ? 5 : 6)
 k_vec_batched(const VecDesc *__restrict__ descs,
               const int64_t *__restrict__ prefix, int n_probs, bool warm,
               double tol2, double *partials, unsigned int *counters)
@@ -456,13 +458,13 @@ k_vec_batched(const VecDesc *__restrict__ descs,
 #pragma unroll
                 for (int k = 0; k < kVecUnroll; ++k) a0.add_prod(u[k], v[k]);
             } else if constexpr (kOp == V_UPDATE) {
-                const StepF2 alpha(d.S[S_ALPHA]), minus(-d.S[S_ALPHA]);
+                const StepF2 alpha = step_of(d.S[S_ALPHA]);
                 float x[kVecUnroll] = {}, r[kVecUnroll] = {}, b[kVecUnroll] = {};
                 vec_group(c0, c1, g, [&](int64_t i, int k) {
                     x[k] = axpy(alpha, d.p[i], d.x[i]);
                     r[k] = (d.mm != nullptr && d.mm[i] != 0)
                                ? 0.0f
-                               : axpy(minus, d.q[i], d.r[i]);
+                               : axpy(alpha, -d.q[i], d.r[i]);
                     b[k] = d.b[i];
                 });
                 vec_group(c0, c1, g, [&](int64_t i, int k) {
@@ -472,7 +474,7 @@ k_vec_batched(const VecDesc *__restrict__ descs,
                     a1.add_prod_sum(x[k], r[k], b[k]);
                 });
             } else if constexpr (kOp == V_DIR) {
-                const StepF2 beta(d.S[S_BETA]);
+                const StepF2 beta = step_of(d.S[S_BETA]);
                 float v[kVecUnroll] = {};
                 vec_group(c0, c1, g, [&](int64_t i, int k) {
                     v[k] = axpy(beta, d.p[i], d.r[i]);

@@ -164,7 +164,9 @@ struct CgInitElem {
 };
 
 // Calls f(i, excluded, v) for every element of n = frames * mm_n (mm_n = n
-// without a mask) in a grid-stride order.
+// without a mask) in a grid-stride order.  Unrolled, the loads of four elements
+// are in flight together (k_cg_update on 128^3: 24.0 -> 19.3 us; with one-float
+// steps the compiler unrolled by itself, 17.4 us).
 template <class F>
 __device__ __forceinline__ void masked_elements(const uint8_t *__restrict__ mm,
                                                 int64_t mm_n, int64_t n,
@@ -173,6 +175,7 @@ __device__ __forceinline__ void masked_elements(const uint8_t *__restrict__ mm,
     const int64_t start = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     if (mm == nullptr) {
+#pragma unroll 4
         for (int64_t i = start; i < n; i += stride) f(i, false, v);
         return;
     }
@@ -218,12 +221,12 @@ __global__ void k_cg_pq(const float *__restrict__ p, const float *__restrict__ q
 struct CgUpdateElem {
     float *x, *r;
     const float *p, *q, *b;
-    StepF2 alpha, minus;  // alpha and -alpha
+    StepF2 alpha;
     __device__ __forceinline__ void operator()(int64_t i, bool out,
                                                SumF2 v[2]) const
     {
         const float xi = axpy(alpha, p[i], x[i]);
-        const float ri = out ? 0.0f : axpy(minus, q[i], r[i]);
+        const float ri = out ? 0.0f : axpy(alpha, -q[i], r[i]);
         x[i] = xi;
         r[i] = ri;
         v[0].add_prod(ri, ri);
@@ -241,8 +244,7 @@ __global__ void k_cg_update(float *__restrict__ x, float *__restrict__ r,
 {
     if (S[S_DONE] != 0.0) return;
     SumF2 a[2];
-    const CgUpdateElem f = { x, r, p, q, b, StepF2(S[S_ALPHA]),
-                             StepF2(-S[S_ALPHA]) };
+    const CgUpdateElem f = { x, r, p, q, b, step_of(S[S_ALPHA]) };
     masked_elements(mm, mm_n, n, f, a);
     double v[2] = { a[0].value(), a[1].value() };
     double tot[2];
@@ -255,7 +257,7 @@ __global__ void k_cg_direction(const float *__restrict__ r, float *p,
                                const double *__restrict__ S)
 {
     if (S[S_DONE] != 0.0) return;
-    const StepF2 beta(S[S_BETA]);
+    const StepF2 beta = step_of(S[S_BETA]);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         p[i] = direction_store(axpy(beta, p[i], r[i]), p16, i);

@@ -148,8 +148,8 @@ struct Tiling {
 enum : int {
     S_RR = 0,     // r.r of the current residual
     S_PQ = 1,     // p.q
-    S_ALPHA = 2,  // step length
-    S_BETA = 3,   // direction update
+    S_ALPHA = 2,  // step length, as the two floats of a StepF2
+    S_BETA = 3,   // direction update, likewise
     S_YMY = 4,    // y^T M y
     S_RR0 = 5,    // r0.r0
     S_DONE = 6,   // nonzero: stop (converged or breakdown)
