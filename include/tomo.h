@@ -45,7 +45,8 @@
  *  - Errors: every entry point validates its arguments before any launch
  *    and returns a tomo_status; it never aborts.  tomo_last_error() gives a
  *    one-line message.  A context must not be used by two host threads at
- *    once.
+ *    once.  Its calls share its workspace: calls on different streams must be
+ *    ordered by the caller (events, or a synchronisation).
  */
 #ifndef TOMO_H
 #define TOMO_H
@@ -143,7 +144,8 @@ typedef struct tomo_ctx tomo_ctx;
                                   ~1 degree of a cube-axis plane, or pixels
                                   at least 0.75 voxel apart (or less, see
                                   fwd_min_pitch in tomo_plane_rules; per ray
-                                  on the others).  A set bit makes the rays of a warp walk the cube one
+                                  on the others).  A set bit makes the rays of
+                                  a warp walk the cube one
                                   plane of the image's major axis at a time,
                                   on a copy of the cube stored with the
                                   image's lateral axis fastest, so the voxels

@@ -277,12 +277,13 @@ k_to_layout_batched(const LayoutJob *__restrict__ jobs,
 // one problem's cube and layout copies.  A CTA covers 32 x 8 pixels of one
 // image; when the image's hint selects the plane forward the warps walk
 // plane by plane on the layout copies, with the gather bodies free of slot
-// predicates and six slabs of loads in flight as in the single-problem
-// forward (irregular lanes per ray on the native cube), otherwise every
-// lane walks its own ray.  Measured on the 32-problem workload: 10.34 ms
-// per projection against 11.0 for a persistent work-queue kernel (whose
-// loop state left no registers for the predicate-free bodies) and 10.29
-// for the single-problem calls one after another.
+// predicates (irregular lanes per ray on the native cube), otherwise every
+// lane walks its own ray.  Voxels go by 32-bit offset, with six slabs of
+// loads in flight in 64 registers (a walk by address needs every problem's
+// cube and copies between two multiples of 2^32).  When it came, 10.34
+// ms per projection of the 32-problem workload against 11.0 for a persistent
+// work-queue kernel, whose loop state left no registers for the predicate-free
+// bodies.
 __global__ void __launch_bounds__(kThreads, 4)
 k_forward_plane_batched(const WalkDesc *__restrict__ descs,
                         const int64_t *__restrict__ prefix, int n_probs)

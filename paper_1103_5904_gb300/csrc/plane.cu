@@ -56,7 +56,9 @@ namespace {
 // four 6.40, three 6.80; six CTAs with four slabs 6.38, with three 7.24; four
 // CTAs with six slabs 6.45); of a bf16 cube (512^3, 48 views of 1024^2) four
 // slabs at six CTAs: 12.53 ms (five CTAs with four to eight slabs
-// 12.94-13.14).  By offset, for a buffer across a multiple of 2^32: 6.92 and
+// 12.94-13.14), although 48 bytes spill from its 40 registers (256^3, 240 views of
+// 512^2: 6.58 ms, float 6.29; widening a bf16 voxel costs an instruction, and L2 holds
+// the float cube too).  By offset, for a buffer across a multiple of 2^32: 6.92 and
 // 14.2 ms at four CTAs with five and six slabs.  The transpose, bound by the
 // rate at which an SM sends reduction sectors to L2, walks one slab per
 // iteration at six CTAs (9.19 ms; five CTAs 9.31, two slabs per iteration

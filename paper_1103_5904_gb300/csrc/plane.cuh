@@ -32,10 +32,11 @@ __device__ __forceinline__ bool plane_cta(int n_img, int group, int &img,
 // axes, a1 the one with the smaller crossing spacing (crossed more often).
 // Voxel positions are byte offsets from the walked buffer's base, held as
 // unsigned 32-bit numbers (a step in the negative direction adds the
-// stride's two's complement, which wraps to the right offset); a gather or
-// reduction then needs no 64-bit index arithmetic, only the base plus a
-// 32-bit offset.  The walked buffer (one cube or one frame pair of it) must
-// therefore span at most 2^32 bytes: plane_supported() checks that.
+// stride's two's complement, which wraps to the right offset), so the walk's
+// state steps in 32 bits and a gather or reduction adds the offset to the base
+// (walks by address step an address instead, see near_step).  The walked buffer
+// (one cube or one frame pair of it) must therefore span at most 2^32 bytes:
+// plane_supported() checks that.
 struct PlaneRay {
     float t0M, t01, t02;  // first crossings
     float AM, A1, A2;     // crossing spacings
@@ -235,14 +236,14 @@ __device__ __forceinline__ void slab_fast_g(const PlaneRay &p, PlaneState &s,
 }
 
 // Adds s (only when on) to the low half of an address.  A gather at base +
-// 32-bit offset costs three more instructions than the load (counted per
-// opcode: two integer additions and a carry), and the walks are bound by
-// instruction issue.  The buffers of a near walk do not cross a multiple of
-// 2^32 (near_buffers), so the high half of an address never changes and a
-// step costs one 32-bit addition, under a predicate for a crossing.  P on
-// the 256^3 cube (240 views of 512^2): 28 -> 22 instructions per slab of a
-// warp, 6.92 -> 6.30 ms; bf16 512^3 (48 of 1024^2) 14.2 -> 12.5 ms.  (One
-// wide multiply-add per gather instead was 19 % slower than the additions.)
+// 32-bit offset forms a 64-bit address for every load, and the walks are
+// bound by instruction issue and load latency.  The buffers of a near walk do
+// not cross a multiple of 2^32 (near_buffers), so the high half of an address
+// never changes and a step costs one 32-bit addition, under a predicate for a
+// crossing.  P on the 256^3 cube (240 views of 512^2) 6.92 -> 6.30 ms (of 24
+// views, with the slot ends above, 7.89e8 -> 6.29e8 warp instructions); bf16
+// 512^3 (48 of 1024^2) 14.2 -> 12.5 ms.  (One wide multiply-add per gather
+// instead was 19 % slower than the additions.)
 __device__ __forceinline__ void near_step(const char *&p, uint32_t s)
 {
     asm("{\n\t.reg .b32 l, h;\n\t"

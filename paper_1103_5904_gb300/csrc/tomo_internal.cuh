@@ -73,10 +73,11 @@ constexpr double kPlaneMinPitch = 0.16;
 //    voxels and more from kPlaneFwdMinPitchLarge on, when a row of voxels is a
 //    whole number of kRowBytes.  The lanes of a per-ray warp read several rows
 //    of the cube at about the same x; with such rows they meet in the same L1
-//    banks (L1 data pipe busy 91-94 % of the time on 128^3 and 160^3 float and
-//    192^3 bf16, 40 % on 132^3), and the per-ray walk takes 1.2 to 1.5x its
-//    time on cubes a few voxels wider.  Per-ray over plane time (by address) at 2 and 7 degrees of
-//    latitude, pixels 0.5 / 0.6 / 0.74 voxel apart:
+//    banks (L1 data pipe busy 87-92 % of the time on 128^3 and 160^3 float and
+//    192^3 bf16, 39-57 % on 132^3 and 168^3 float and 200^3 bf16), and a
+//    per-ray segment takes 1.2 to 1.3 times as long there.  Per-ray over plane
+//    time (by address) at 2 and 7 degrees of latitude, pixels 0.5 / 0.6 / 0.74
+//    voxel apart:
 //      float  128^3 1.10 1.16 / 1.25 1.31 / 1.30 1.36, 160^3 1.18 1.20 / 1.31
 //      1.36 / 1.42 1.58, 256^3 1.30 1.37 / 1.38 1.46 / 1.37 1.47; but 132^3
 //      0.94 1.00 / 0.93 0.99 / 0.90 0.96, 200^3 0.97 1.04 / 0.98 1.05 / 0.97
